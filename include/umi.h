@@ -123,7 +123,7 @@ umi_status umi_detrend(const float *flux_d, int64_t n, int32_t W, const umi_para
  *   W_h        [B] host array of odd window lengths, one per curve
  *   B          number of curves, >= 0
  *   params     shared by all curves; NULL means defaults
- * Device scratch (the work queue, a few bytes per tile) comes from the
+ * Device scratch (the work queue, 60 bytes per curve) comes from the
  * stream-ordered allocator (cudaMallocAsync) on `stream` and is released on
  * the same stream.  Asynchronous on `stream`.  Equal-shaped batches of two or
  * more curves replay a cached CUDA graph (see umi_set_graph_cache); a batch
@@ -170,7 +170,7 @@ umi_status umi_detrend_batched_host(const float *flux_h, const int64_t *offsets_
  * may synchronise the device and block for an unbounded time), or a
  * deployment where the stream-ordered memory pool is disabled.  This call
  * runs the same batched work-queue kernel, but its work-queue tables (curve
- * descriptors, tile items, counters) live in one file-scope device array of
+ * descriptors, first tiles, counters) live in one file-scope device array of
  * UMI_NOALLOC_SCRATCH_BYTES (4 MiB) that every GPU loading libumi holds until
  * the process exits.  The caller still passes the input and output buffers.
  *   - It calls no cudaMalloc, cudaMallocAsync, cudaFree or other device
@@ -180,15 +180,14 @@ umi_status umi_detrend_batched_host(const float *flux_h, const int64_t *offsets_
  *     detrend; a launch copies its parameters when it is enqueued, so the
  *     call does not wait for earlier work on `stream` and returns at once.
  *   - A batch whose tables need more than UMI_NOALLOC_SCRATCH_BYTES returns
- *     UMI_ERR_INVALID_ARG with the size in umi_last_error(); 56 bytes per
- *     curve plus 8 bytes per tile, and a tile covers 288 to 544 positions at
- *     W = 361 depending on the plan (roughly 7,500 to 12,000 curves of
- *     18,000 samples); split larger batches.
+ *     UMI_ERR_INVALID_ARG with the size in umi_last_error(); 60 bytes per
+ *     curve of any length plus 4 bytes per window length (about 69,000
+ *     curves); split larger batches.
  *   - The first call on each device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current; make that first call
  *     before any stream capture.
  *   - Every call shares the one array, which keeps the last call's tables;
- *     each call rewrites the tables and clears its counters on `stream`
+ *     each call rewrites the tables and counters on `stream`
  *     before its kernels run.  Calls whose work overlaps on the GPU (for
  *     example on two streams at once) race on the array: order them on one
  *     stream or serialise them.
@@ -251,7 +250,9 @@ int32_t umi_max_window(void);
  * per lane group, `threads` = threads per CTA, `latency` = 1 when the band is
  * too small to fill the GPU at the shortest chain of the throughput variant
  * (then a 32-lane variant is used where one covers W within 2W, so that
- * every window can start its own chain).
+ * every window can start its own chain).  `chain` is the rule's for a band of
+ * that size; a launch of a plan that was not tuned fits it to its own curves,
+ * which changes its speed and no result.
  *
  * Every call plans each band from its own size, so the same curve can run on
  * different variants alone and inside a large batch.  Variants differ only in

@@ -190,6 +190,7 @@ umi_status launch_single_curve(const Curve &c, int64_t plan_positions, const Dia
     Plan plan;
     umi_status st = make_plan(c.W, plan_positions, &plan);
     if (st != UMI_OK) return st;
+    fit_launch(c.n, 1, &plan);
     const int flavour = (diag ? kFlagDiag : 0) | (c.scale_mode == UMI_SCALE_MAD ? kFlagMad : 0);
     st = prepare_kernel(plan, flavour);
     if (st != UMI_OK) return st;
@@ -200,7 +201,6 @@ umi_status launch_single_curve(const Curve &c, int64_t plan_positions, const Dia
     memset(&a, 0, sizeof(a));
     a.curves = nullptr;
     a.single = c;
-    a.items = nullptr;
     a.n_items = (int32_t)items;
     a.chain = plan.chain;
     a.queue = nullptr;
@@ -254,58 +254,82 @@ umi_status build_layout(const std::vector<Curve> &curves, BatchLayout *layout,
             if (it != plan_sizes->end()) kv.second = std::max(kv.second, it->second);
         }
     std::map<std::tuple<int, int, int, int, int>, std::vector<int>> by_plan;
-    std::vector<Plan> plans;
+    std::map<std::pair<int, int>, Plan> plans;  // one per (window length, scale mode)
     for (size_t b = 0; b < curves.size(); ++b) {
-        Plan p;
-        umi_status st =
-            make_plan(curves[b].W, band_positions[std::make_pair(curves[b].W, curves[b].scale_mode)], &p);
-        if (st != UMI_OK) return st;
+        const auto key = std::make_pair(curves[b].W, curves[b].scale_mode);
+        auto it = plans.find(key);
+        if (it == plans.end()) {
+            Plan p;
+            umi_status st = make_plan(curves[b].W, band_positions[key], &p);
+            if (st != UMI_OK) return st;
+            it = plans.emplace(key, p).first;
+        }
+        const Plan &p = it->second;
         const int flavour = curves[b].scale_mode == UMI_SCALE_MAD ? kFlagMad : 0;
-        by_plan[std::make_tuple(-p.G * p.R, p.variant, p.chain, p.threads, flavour)].push_back((int)b);
-        plans.push_back(p);
+        // Untuned plans of one variant share a launch, whose chain is fitted below.
+        by_plan[std::make_tuple(-p.G * p.R, p.variant, p.tuned ? p.chain : 0, p.threads, flavour)]
+            .push_back((int)b);
     }
     layout->bands.clear();
-    layout->items.clear();
-    layout->n_curves = (int32_t)curves.size();
+    layout->curves.clear();
+    layout->first_tile.clear();
+    std::vector<Curve> cs;
     for (auto &kv : by_plan) {
-        BatchLayout::Band band;
-        band.plan = plans[kv.second.front()];
-        band.flavour = std::get<4>(kv.first);
-        band.first_item = (int32_t)layout->items.size();
-        const int64_t T = band.plan.tile();
         // Longest curves first: their tiles are interleaved with others by the
         // queue anyway, but this keeps the tail short.
         std::vector<int> order = kv.second;
         std::stable_sort(order.begin(), order.end(),
                          [&](int a, int b) { return curves[a].n > curves[b].n; });
-        for (int b : order) {
-            const int64_t tiles = (curves[b].n + T - 1) / T;
-            for (int64_t k = 0; k < tiles; ++k) {
-                if (layout->items.size() >= (size_t)INT32_MAX)
-                    return fail(UMI_ERR_INVALID_ARG, "too many work items");
-                layout->items.push_back(Item{(int32_t)b, (int32_t)k});
-            }
-        }
-        band.n_items = (int32_t)layout->items.size() - band.first_item;
-        if (band.n_items > 0) layout->bands.push_back(band);
+        cs.clear();
+        for (int b : order) cs.push_back(curves[b]);
+        int64_t positions = 0;
+        for (const Curve &c : cs) positions += c.n;
+        Plan plan = plans[std::make_pair(cs.front().W, cs.front().scale_mode)];
+        fit_launch(positions, (int64_t)cs.size(), &plan);
+        umi_status st = layout->add_band(plan, std::get<4>(kv.first), cs);
+        if (st != UMI_OK) return st;
     }
     return UMI_OK;
 }
 
-// Device scratch for one batch: [curve table][items][one counter per band].
-struct Scratch {
-    size_t curve_off = 0, item_off = 0, counter_off = 0, bytes = 0;
-};
+umi_status BatchLayout::add_band(const Plan &plan, int flavour, const std::vector<Curve> &cs)
+{
+    Band band;
+    band.plan = plan;
+    band.flavour = flavour;
+    band.first_curve = (int32_t)curves.size();
+    const int64_t T = plan.tile();
+    int64_t items = 0;
+    for (const Curve &c : cs) {
+        if (c.n <= 0) continue;  // every curve of the table owns at least one item
+        curves.push_back(c);
+        first_tile.push_back((int32_t)items);
+        items += (c.n + T - 1) / T;
+        if (items > INT32_MAX) return fail(UMI_ERR_INVALID_ARG, "too many work items");
+    }
+    band.n_curves = (int32_t)curves.size() - band.first_curve;
+    band.n_items = (int32_t)items;
+    if (band.n_items > 0) bands.push_back(band);
+    return UMI_OK;
+}
 
-static Scratch scratch_layout(size_t n_curves, size_t n_items, size_t n_bands)
+static Scratch scratch_layout(const BatchLayout &lay)
 {
     Scratch s;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     s.curve_off = 0;
-    s.item_off = up(n_curves * sizeof(Curve));
-    s.counter_off = s.item_off + up(n_items * sizeof(Item));
-    s.bytes = s.counter_off + up(std::max<size_t>(1, n_bands) * sizeof(int32_t));
+    s.tile_off = up(lay.curves.size() * sizeof(Curve));
+    s.counter_off = s.tile_off + up(lay.curves.size() * sizeof(int32_t));
+    s.bytes = s.counter_off + up(std::max<size_t>(1, lay.bands.size()) * sizeof(uint32_t));
     return s;
+}
+
+// Host image of the scratch: tables and zeroed counters.
+static void write_tables(const BatchLayout &lay, const Scratch &sc, char *host)
+{
+    memcpy(host + sc.curve_off, lay.curves.data(), lay.curves.size() * sizeof(Curve));
+    memcpy(host + sc.tile_off, lay.first_tile.data(), lay.first_tile.size() * sizeof(int32_t));
+    memset(host + sc.counter_off, 0, sc.bytes - sc.counter_off);
 }
 
 static umi_status enqueue_bands(const BatchLayout &lay, char *dev, const Scratch &sc,
@@ -313,19 +337,17 @@ static umi_status enqueue_bands(const BatchLayout &lay, char *dev, const Scratch
 {
     int nv = 0;
     const Variant *t = variant_table(&nv);
-    UMI_CUDA(cudaMemsetAsync(dev + sc.counter_off, 0, lay.bands.size() * sizeof(int32_t), stream),
-             "cudaMemsetAsync");
     int count = 0;
     for (size_t k = 0; k < lay.bands.size(); ++k) {
         const BatchLayout::Band &band = lay.bands[k];
         LaunchArgs a;
         memset(&a, 0, sizeof(a));
-        a.curves = reinterpret_cast<const Curve *>(dev + sc.curve_off);
-        a.items = reinterpret_cast<const Item *>(dev + sc.item_off) + band.first_item;
+        a.curves = reinterpret_cast<const Curve *>(dev + sc.curve_off) + band.first_curve;
+        a.first_tile = reinterpret_cast<const int32_t *>(dev + sc.tile_off) + band.first_curve;
         a.n_items = band.n_items;
         a.chain = band.plan.chain;
-        a.queue = reinterpret_cast<int32_t *>(dev + sc.counter_off) + k;
-        a.n_curves = lay.n_curves;
+        a.queue = reinterpret_cast<uint32_t *>(dev + sc.counter_off) + k;
+        a.n_curves = band.n_curves;
         a.check = check_word();
         const int warps = band.plan.threads / 32;
         const int grid =
@@ -347,29 +369,18 @@ umi_status prepare_batch(const std::vector<Curve> &curves, PreparedBatch *pb)
         st = prepare_kernel(band.plan, band.flavour);
         if (st != UMI_OK) return st;
     }
-    const Scratch sc = scratch_layout(curves.size(), pb->layout.items.size(), pb->layout.bands.size());
-    pb->curve_off = sc.curve_off;
-    pb->item_off = sc.item_off;
-    pb->counter_off = sc.counter_off;
-    pb->dev_bytes = sc.bytes;
-    pb->host_bytes = sc.counter_off;
+    pb->scratch = scratch_layout(pb->layout);
     return UMI_OK;
 }
 
-umi_status enqueue_prepared(const std::vector<Curve> &curves, const PreparedBatch &pb, char *dev,
-                            char *host, cudaStream_t stream, int *launches)
+umi_status enqueue_prepared(const PreparedBatch &pb, char *dev, char *host, cudaStream_t stream,
+                            int *launches)
 {
     if (launches) *launches = 0;
-    if (pb.layout.items.empty()) return UMI_OK;
-    memcpy(host + pb.curve_off, curves.data(), curves.size() * sizeof(Curve));
-    memcpy(host + pb.item_off, pb.layout.items.data(), pb.layout.items.size() * sizeof(Item));
-    UMI_CUDA(cudaMemcpyAsync(dev, host, pb.host_bytes, cudaMemcpyHostToDevice, stream), "cudaMemcpyAsync");
-    Scratch sc;
-    sc.curve_off = pb.curve_off;
-    sc.item_off = pb.item_off;
-    sc.counter_off = pb.counter_off;
-    sc.bytes = pb.dev_bytes;
-    return enqueue_bands(pb.layout, dev, sc, stream, launches);
+    if (pb.layout.bands.empty()) return UMI_OK;
+    write_tables(pb.layout, pb.scratch, host);
+    UMI_CUDA(cudaMemcpyAsync(dev, host, pb.scratch.bytes, cudaMemcpyHostToDevice, stream), "cudaMemcpyAsync");
+    return enqueue_bands(pb.layout, dev, pb.scratch, stream, launches);
 }
 
 // Pinned host staging for work-queue tables: a ring of a few buffers per
@@ -487,23 +498,22 @@ umi_status launch_curve_table(const std::vector<Curve> &curves, cudaStream_t str
     BatchLayout lay;
     umi_status st = build_layout(curves, &lay, plan_sizes);
     if (st != UMI_OK) return st;
-    if (lay.items.empty()) return UMI_OK;
+    if (lay.bands.empty()) return UMI_OK;
     for (const auto &band : lay.bands) {
         st = prepare_kernel(band.plan, band.flavour);
         if (st != UMI_OK) return st;
     }
-    const Scratch sc = scratch_layout(curves.size(), lay.items.size(), lay.bands.size());
+    const Scratch sc = scratch_layout(lay);
     keep_pool_memory();
     // Host staging in one pinned block so a single asynchronous copy moves the tables.
     int slot = 0;
     char *host = nullptr;
-    st = acquire_pinned(sc.counter_off, &slot, &host);
+    st = acquire_pinned(sc.bytes, &slot, &host);
     if (st != UMI_OK) return st;
-    memcpy(host + sc.curve_off, curves.data(), curves.size() * sizeof(Curve));
-    memcpy(host + sc.item_off, lay.items.data(), lay.items.size() * sizeof(Item));
+    write_tables(lay, sc, host);
     void *dev = nullptr;
     UMI_CUDA(cudaMallocAsync(&dev, sc.bytes, stream), "cudaMallocAsync");
-    cudaError_t e = cudaMemcpyAsync(dev, host, sc.counter_off, cudaMemcpyHostToDevice, stream);
+    cudaError_t e = cudaMemcpyAsync(dev, host, sc.bytes, cudaMemcpyHostToDevice, stream);
     release_pinned(slot, stream);
     if (e != cudaSuccess) {
         cudaFreeAsync(dev, stream);
@@ -568,14 +578,12 @@ static umi_status build_graph(const std::vector<Curve> &curves, GraphEntry *g)
         if (st != UMI_OK) return st;
     }
     // Batches of two or more curves only (one curve launches directly).
-    const Scratch sc = scratch_layout(curves.size(), lay.items.size(), lay.bands.size());
+    const Scratch sc = scratch_layout(lay);
     {
-        std::vector<char> host(sc.counter_off);
-        memcpy(host.data() + sc.curve_off, curves.data(), curves.size() * sizeof(Curve));
-        if (!lay.items.empty())
-            memcpy(host.data() + sc.item_off, lay.items.data(), lay.items.size() * sizeof(Item));
+        std::vector<char> host(sc.bytes);
+        write_tables(lay, sc, host.data());
         UMI_CUDA(cudaMalloc(&g->dev, sc.bytes), "cudaMalloc (graph tables)");
-        UMI_CUDA(cudaMemcpy(g->dev, host.data(), sc.counter_off, cudaMemcpyHostToDevice), "cudaMemcpy");
+        UMI_CUDA(cudaMemcpy(g->dev, host.data(), sc.bytes, cudaMemcpyHostToDevice), "cudaMemcpy");
     }
     cudaStream_t cs;
     UMI_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -725,25 +733,15 @@ static umi_status time_plan(const Plan &plan, const float *flux, float *trend, f
         o += n;
     }
     BatchLayout lay;
-    lay.n_curves = (int32_t)curves.size();
-    lay.bands.resize(1);
-    lay.bands[0].plan = plan;
-    lay.bands[0].first_item = 0;
-    const int64_t T = plan.tile();
-    for (size_t c = 0; c < lengths.size(); ++c) {
-        const int64_t tiles = (lengths[c] + T - 1) / T;
-        for (int64_t k = 0; k < tiles; ++k) lay.items.push_back(Item{(int32_t)c, (int32_t)k});
-    }
-    lay.bands[0].n_items = (int32_t)lay.items.size();
-    umi_status st = prepare_kernel(plan, 0);
+    umi_status st = lay.add_band(plan, 0, curves);
+    if (st == UMI_OK) st = prepare_kernel(plan, 0);
     if (st != UMI_OK) return st;
-    const Scratch sc = scratch_layout(curves.size(), lay.items.size(), 1);
-    std::vector<char> host(sc.counter_off);
-    memcpy(host.data() + sc.curve_off, curves.data(), curves.size() * sizeof(Curve));
-    memcpy(host.data() + sc.item_off, lay.items.data(), lay.items.size() * sizeof(Item));
+    const Scratch sc = scratch_layout(lay);
+    std::vector<char> host(sc.bytes);
+    write_tables(lay, sc, host.data());
     void *dev = nullptr;
     UMI_CUDA(cudaMalloc(&dev, sc.bytes), "cudaMalloc");
-    UMI_CUDA(cudaMemcpy(dev, host.data(), sc.counter_off, cudaMemcpyHostToDevice), "cudaMemcpy");
+    UMI_CUDA(cudaMemcpy(dev, host.data(), sc.bytes, cudaMemcpyHostToDevice), "cudaMemcpy");
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -855,8 +853,8 @@ static umi_status noalloc_batched(const float *flux, const int64_t *offsets, con
     BatchLayout lay;
     st = build_layout(curves, &lay);
     if (st != UMI_OK) return st;
-    if (lay.items.empty()) return UMI_OK;
-    const Scratch sc = scratch_layout(curves.size(), lay.items.size(), lay.bands.size());
+    if (lay.bands.empty()) return UMI_OK;
+    const Scratch sc = scratch_layout(lay);
     if (sc.bytes > UMI_NOALLOC_SCRATCH_BYTES)
         return fail(UMI_ERR_INVALID_ARG,
                     "batch needs " + std::to_string(sc.bytes) + " bytes of work-queue tables, above the " +
@@ -871,9 +869,8 @@ static umi_status noalloc_batched(const float *flux, const int64_t *offsets, con
     if (st != UMI_OK) return st;
     // Host image of the tables (the scratch layout's offsets are multiples of
     // 256 bytes, so it is a whole number of words).
-    std::vector<uint32_t> host(sc.counter_off / sizeof(uint32_t));
-    memcpy((char *)host.data() + sc.curve_off, curves.data(), curves.size() * sizeof(Curve));
-    memcpy((char *)host.data() + sc.item_off, lay.items.data(), lay.items.size() * sizeof(Item));
+    std::vector<uint32_t> host(sc.bytes / sizeof(uint32_t));
+    write_tables(lay, sc, (char *)host.data());
     // Stream-ordered after any earlier call's kernels on this stream.
     std::unique_ptr<TableChunk> chunk(new TableChunk);
     int writers = 0;
@@ -892,7 +889,7 @@ static umi_status noalloc_batched(const float *flux, const int64_t *offsets, con
         ++writers;
     }
     int launches = 0;
-    st = enqueue_bands(lay, (char *)dev, sc, stream, &launches);  // clears the counters first
+    st = enqueue_bands(lay, (char *)dev, sc, stream, &launches);
     g_kernel_launches += writers + launches;
     return st;
 }

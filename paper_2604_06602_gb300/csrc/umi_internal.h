@@ -41,6 +41,7 @@ struct Plan {
     int chain = 0;    // positions per group
     int threads = 0;  // per CTA
     int regime = 0;   // kRegimeThroughput or kRegimeLatency
+    bool tuned = false;    // from the tuner or a tuning file, else from the rule
     int64_t tuned_at = 0;  // band size a tuned plan was measured at (0: unknown)
     // Positions per work item (one warp's tile).
     int tile() const { return (32 / G) * chain; }
@@ -67,6 +68,9 @@ int plan_regime(int W, int64_t positions);
 // large enough for the longest chain): the tuned plan for (W, regime) if any,
 // else the measured rule; the chain shrinks for small bands.
 umi_status make_plan(int W, int64_t positions, Plan *plan);
+// Sets the chain of a launch over `n_curves` curves with `positions` windows in
+// all (results do not depend on it).  Tuned plans keep theirs.
+void fit_launch(int64_t positions, int64_t n_curves, Plan *plan);
 // The plans umi_autotune times for a band of `positions` windows of length W.
 std::vector<Plan> autotune_candidates(int W, int64_t positions);
 // Records a tuned plan for (W, p.regime).
@@ -122,33 +126,42 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
                              const umi_params *params, const umi_segment_params *seg, float *trend,
                              float *detr, int64_t *segments_out, cudaStream_t stream);
 
-// Work-item list and per-variant launch layout for a curve table.
+// Launch layout of a curve table: the curves permuted so that each band's are
+// consecutive, and each curve's first work item within its band.
 struct BatchLayout {
     struct Band {
         Plan plan;
         int flavour = 0;  // kFlagMad when the band's curves use the MAD scale
-        int32_t first_item = 0;
+        int32_t first_curve = 0;
+        int32_t n_curves = 0;
         int32_t n_items = 0;
     };
     std::vector<Band> bands;
-    std::vector<Item> items;
-    int32_t n_curves = 0;  // entries of the curve table the items index
+    std::vector<Curve> curves;
+    std::vector<int32_t> first_tile;
+    // Appends a band over `cs` and numbers its tiles.
+    umi_status add_band(const Plan &plan, int flavour, const std::vector<Curve> &cs);
 };
 umi_status build_layout(const std::vector<Curve> &curves, BatchLayout *layout,
                         const BandSizes *plan_sizes = nullptr);
 
-// A batch planned for caller-owned buffers: `dev_bytes` of device scratch and
-// `host_bytes` of (preferably pinned) host staging for the tables.
+// Device scratch for one batch: [curve table][first tiles][one counter per
+// band], all of it written by the host.
+struct Scratch {
+    size_t curve_off = 0, tile_off = 0, counter_off = 0, bytes = 0;
+};
+
+// A batch planned for caller-owned buffers: scratch.bytes of device memory and
+// as much (preferably pinned) host staging for the tables.
 struct PreparedBatch {
     BatchLayout layout;
-    size_t curve_off = 0, item_off = 0, counter_off = 0;
-    size_t dev_bytes = 0, host_bytes = 0;
+    Scratch scratch;
 };
 umi_status prepare_batch(const std::vector<Curve> &curves, PreparedBatch *pb);
-// Stages the tables in `host`, copies them to `dev` on `stream`, clears the
-// counters and launches the bands.  The host buffer must stay untouched until
+// Stages the tables in `host`, copies them to `dev` on `stream` and launches
+// the bands.  The host buffer must stay untouched until
 // the copy has run (stream order).
-umi_status enqueue_prepared(const std::vector<Curve> &curves, const PreparedBatch &pb, char *dev,
-                            char *host, cudaStream_t stream, int *launches);
+umi_status enqueue_prepared(const PreparedBatch &pb, char *dev, char *host, cudaStream_t stream,
+                            int *launches);
 
 }  // namespace umi

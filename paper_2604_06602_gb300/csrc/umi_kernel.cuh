@@ -16,8 +16,8 @@
 //    slots past W hold kGap).  The 32/G groups of a warp run in lock step on
 //    neighbouring chains; every block that shuffles is entered warp-uniformly.
 //  * Each group walks a chain of P consecutive positions.  At the chain start
-//    (or after an empty window) the median comes from an exact binary search
-//    over order-preserving integer keys.  Afterwards the group keeps the
+//    (or after an empty window) the median comes from an exact rank select
+//    over the registers.  Afterwards the group keeps the
 //    counts L = #{x < m}, E = #{x == m}, G+ = #{x > m} of the current window
 //    and updates them in O(1) per step from the sample that leaves and the one
 //    that enters.  One step moves the median's rank by at most one, so the new
@@ -67,20 +67,19 @@ struct Diag {
     float *scale;
 };
 
-struct Item {
-    int32_t curve;  // index into the curve table
-    int32_t tile;   // tile index within the curve; first position = tile * T
-};
-
+// A work item is one tile of T = (32/G)*P positions of one curve.  Items are
+// numbered through the launch's curves: curve c owns the items first_tile[c]
+// .. first_tile[c + 1] - 1 (the last one up to n_items - 1).
 struct LaunchArgs {
-    const Curve *curves;  // device curve table, or nullptr to use `single`
+    const Curve *curves;  // device curve table of the launch, or nullptr to use `single`
     Curve single;
-    const Item *items;    // device item list, or nullptr: item i = {0, i}
+    const int32_t *first_tile;  // [n_curves], ascending from 0 (unused with `single`)
     int32_t n_items;
     int32_t chain;        // P: consecutive positions per group
-    int32_t *queue;       // persistent work counter, or nullptr: one item per CTA
+    uint32_t *queue;      // persistent work counter (0 between launches), or
+                          // nullptr: one item per warp
     Diag diag;
-    int32_t n_curves;     // entries of `curves` (checked builds test item indices)
+    int32_t n_curves;     // entries of `curves`
     uint32_t *check;      // checked builds: flag word of failed index checks
 };
 
@@ -91,7 +90,7 @@ struct LaunchArgs {
 enum : uint32_t {
     kCheckSmemSize = 1u << 0,    // the warps' tile slices exceed the launch's dynamic smem
     kCheckTileRead = 1u << 1,    // window, slide or centre read outside the warp's tile
-    kCheckCurveIndex = 1u << 2,  // work item names a curve outside the table
+    kCheckCurveIndex = 1u << 2,  // work item found no curve, or one outside the table
     kCheckItemTile = 1u << 3,    // work item's tile starts past its curve's end
 };
 
@@ -693,10 +692,32 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
     }
 }
 
+// The curve that owns work item `item`: the last c with first_tile[c] <= item,
+// by a warp-wide search that divides the range by 32 per round (two dependent
+// loads for 1000 curves).  A table of items instead, 8 bytes per tile written
+// by the host and copied before the launch, was 0.5 MB for 1000 curves of
+// 18,000 samples, and grew with every shorter chain.
+__device__ __forceinline__ int find_curve(const int32_t *__restrict__ first_tile, int n, int item, int lane)
+{
+    int lo = 0, len = n;
+    while (len > 1) {
+        const int step = (len + 31) >> 5;
+        const int at = lane * step;
+        const bool below = at < len && first_tile[lo + at] <= item;
+        const int k = max(__popc(__ballot_sync(0xffffffffu, below)) - 1, 0);
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    return lo;
+}
+
 // Work items belong to warps: each warp stages its own tile of T = (32/G)*P
 // positions (plus the S-1 halo samples) in its slice of shared memory, so no
 // CTA-wide barrier is ever needed.  Without a queue, warp w of CTA b takes
 // item b*warps + w; with a queue, each warp pulls items until none is left.
+// Every warp makes exactly one pull past the end, so the counter's wrap value
+// brings it back to 0 with the launch's last pull and the next launch needs
+// no memset before it.
 // Dynamic shared memory: warps * (T + S - 1) floats, plus warps * T for the
 // staged trend when stages_outputs(G).  MINB (CTAs of 256
 // threads per SM) sets the register budget the compiler aims for.  FLAGS
@@ -736,23 +757,27 @@ __global__ void __launch_bounds__(256, MINB) umi_tile_kernel(LaunchArgs a)
     for (;;) {
         if (a.queue) {
             int v = 0;
-            if (lane == 0) v = atomicAdd(a.queue, 1);
+            if (lane == 0) v = (int)atomicInc(a.queue, (unsigned)a.n_items + gridDim.x * n_warps - 1u);
             item = __shfl_sync(0xffffffffu, v, 0);
         }
         if (item >= a.n_items) break;
-        const Item wi = a.items ? a.items[item] : Item{0, item};
+        int curve = 0, tile_idx = item;
+        if (a.curves) {
+            curve = find_curve(a.first_tile, a.n_curves, item, lane);
 #ifdef UMI_CHECKED
-        if (a.curves && (wi.curve < 0 || wi.curve >= a.n_curves)) {
-            if (lane == 0 && a.check) atomicOr(a.check, kCheckCurveIndex);
-            if (!a.queue) break;
-            continue;
-        }
+            if (curve < 0 || curve >= a.n_curves) {
+                if (lane == 0 && a.check) atomicOr(a.check, kCheckCurveIndex);
+                if (!a.queue) break;
+                continue;
+            }
 #endif
-        const Curve cv = a.curves ? a.curves[wi.curve] : a.single;
-        const int64_t t0 = (int64_t)wi.tile * T;
+            tile_idx -= a.first_tile[curve];
+        }
+        const Curve cv = a.curves ? a.curves[curve] : a.single;
+        const int64_t t0 = (int64_t)tile_idx * T;
         const int h = (cv.W - 1) >> 1;
 #ifdef UMI_CHECKED
-        if (wi.tile < 0 || t0 >= (cv.n > 0 ? cv.n : 1)) {
+        if (tile_idx < 0 || t0 >= (cv.n > 0 ? cv.n : 1)) {
             if (lane == 0 && a.check) atomicOr(a.check, kCheckItemTile);
             if (!a.queue) break;
             continue;

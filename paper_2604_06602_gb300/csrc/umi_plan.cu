@@ -191,7 +191,7 @@ umi_status make_plan(int W, int64_t positions, Plan *plan)
         auto it = g_tuned.find(std::make_pair(W, regime));
         if (it != g_tuned.end()) {
             p = it->second;
-            tuned = true;
+            p.tuned = tuned = true;
         }
     }
     if (!tuned) {
@@ -219,6 +219,45 @@ umi_status make_plan(int W, int64_t positions, Plan *plan)
     p.regime = regime;
     *plan = p;
     return UMI_OK;
+}
+
+// A window's result depends on its variant, not on the chain it lies in, so a
+// launch of an untuned plan fits the chain to its own curves.  With N steps
+// (one window per group) for every resident warp, a chain of c steps costs
+//     (tiles per warp) * (c + kStartSteps) + kTailTiles * (c + kStartSteps):
+// each tile stages its samples and selects its first median, about three
+// quarters of a step's work, and the launch ends with a partly idle tile;
+// tiles are whole per curve (half a tile lost in each).  600 curves of 18,000
+// samples at W = 361 (N = 1110): 5.35 ms at a chain of 136, 5.14 at 72, 5.09 at
+// 56, 5.11 at 40; 32 of 118,000 at W = 2161 (N = 1552): 9.65 ms at 136, 9.53 at
+// 48.  Bands of at most G steps per warp take the shortest chain that gives
+// every resident warp one tile (chains up to G are bank-conflict free too):
+// one curve of 18,000 samples at W = 721 43 us at a chain of 16, 33 at 8, 31 at
+// 4, 35 at 2 (two tiles for some warps).
+void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
+{
+    static const double kStartSteps = 0.75, kTailTiles = 0.35;
+    if (plan->tuned) return;
+    int nv = 0;
+    const Variant *t = variant_table(&nv);
+    const int G = plan->G, groups = 32 / G;
+    const int64_t warps = (int64_t)std::max(1, device_info(current_device()).sms) * 8 * t[plan->variant].minb;
+    const int64_t steps = (positions + warps * groups - 1) / (warps * groups);
+    if (steps <= G) {
+        plan->chain = (int)std::max<int64_t>(1, steps);
+        return;
+    }
+    const int cap = chain_cap(G);
+    double best = 1e300;
+    for (int c = chain_at_least(G, 1); c <= cap; c = chain_at_least(G, c + 1)) {
+        const double tiles = (double)positions / (groups * c) + 0.5 * (double)n_curves;
+        const double cost = (std::max(1.0, tiles / (double)warps) + kTailTiles) * (c + kStartSteps);
+        if (cost < best) {
+            best = cost;
+            plan->chain = c;
+        }
+        if (G >= 32 && c >= 16) c += 7;  // a coarser grid is enough there
+    }
 }
 
 // The candidates umi_autotune times for a band: the variants that waste at

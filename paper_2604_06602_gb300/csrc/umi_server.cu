@@ -295,21 +295,21 @@ static void launch_batch_locked(umi_server *s, int k, int32_t W0, std::unique_lo
         StreamBuffers &sb = s->bufs[k];
         // This stream's previous batch has completed (it is idle), so its
         // buffers may be regrown or rewritten.
-        if (ok && pb.dev_bytes > sb.dev_bytes) {
+        if (ok && pb.scratch.bytes > sb.dev_bytes) {
             if (sb.dev) cudaFree(sb.dev);
             sb.dev = nullptr;
             sb.dev_bytes = 0;
-            if (cudaMalloc((void **)&sb.dev, 2 * pb.dev_bytes) == cudaSuccess) sb.dev_bytes = 2 * pb.dev_bytes;
+            if (cudaMalloc((void **)&sb.dev, 2 * pb.scratch.bytes) == cudaSuccess) sb.dev_bytes = 2 * pb.scratch.bytes;
             else ok = false;
         }
-        if (ok && pb.host_bytes > sb.host_bytes) {
+        if (ok && pb.scratch.bytes > sb.host_bytes) {
             if (sb.host) cudaFreeHost(sb.host);
             sb.host = nullptr;
             sb.host_bytes = 0;
-            if (cudaMallocHost((void **)&sb.host, 2 * pb.host_bytes) == cudaSuccess) sb.host_bytes = 2 * pb.host_bytes;
+            if (cudaMallocHost((void **)&sb.host, 2 * pb.scratch.bytes) == cudaSuccess) sb.host_bytes = 2 * pb.scratch.bytes;
             else ok = false;
         }
-        if (ok && enqueue_prepared(curves, pb, sb.dev, sb.host, st, &launches) != UMI_OK) ok = false;
+        if (ok && enqueue_prepared(pb, sb.dev, sb.host, st, &launches) != UMI_OK) ok = false;
     }
     if (ok) {
         const cudaError_t e = s->cfg.busy_poll ? cudaEventRecord(s->done_events[k], st)

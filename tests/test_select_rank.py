@@ -1,5 +1,5 @@
-"""The kernel's rank select (the chain-start median and the MAD) on value
-distributions its pivots can go wrong on, against the oracle: medians, valid
+"""The kernel's rank select (the chain-start median and the MAD) and its rank walk
+along a chain on value distributions they can go wrong on, against the oracle: medians, valid
 counts and above-median counts exactly.  The MAD is an order statistic of
 fl(|x - m|), each one rounding of the exact |x - m| and monotone in it, so it
 is the rounding of the exact MAD: one unit of FP32 (relative 2^-23, or one
@@ -25,6 +25,9 @@ def curves(n, W):
         "powers": np.exp2(rng.integers(-59, 59, n).astype(float)) * rng.choice([-1.0, 1.0], n),
         "negative": -1.0 + noise,
         "around_zero": noise,
+        # Median and neighbours on both sides of zero (the rank walk's two forms).
+        "sign_edge": rng.choice([-1.0, 1.0], n) * rng.uniform(0.5, 2.0, n),
+        "mostly_positive": np.abs(noise) - np.where(rng.random(n) < 0.45, 3e-3, 0.0),
         "levels": 1.0 + 1e-3 * rng.integers(0, 4, n),
         "sparse": np.where(rng.random(n) < 2.5 / W, 1.0 + noise, np.nan),
         "gaps": 1.0 + noise,
