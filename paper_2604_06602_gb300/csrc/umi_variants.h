@@ -63,19 +63,51 @@ const Variant *variant_table(int *count);
 
 // The variant list: (G, R, MINB), ordered by slot capacity G*R; for equal
 // capacity the first entry is the default and the autotuner may pick others.
+// Every slot past W is work for nothing, so the capacities follow each other
+// within about a fifth; and a capacity is cut into as few lanes as 56 to 68
+// slots allow: fewer lanes reduce in fewer steps and serve more windows per
+// warp at the same 16 warps per SM.  ns per window, large bands: W = 73 (2,38)
+// 0.106, (4,20) 0.120, (4,32) 0.176; W = 217 (4,56) 0.289, (8,28) 0.342, (8,46)
+// 0.50; W = 433 (8,56) 0.602, (16,28) 0.653, (16,48) 1.05; W = 2521 (32,96) 4.2,
+// (32,128) 5.4.  (2,32,2) and (4,32,2) are there because small bands take the
+// largest register budget among the near capacities and would otherwise skip
+// to the next one; no 32-lane capacity lies between 721 and 1442, where small
+// bands of W = 721 would take it in place of (16,48,2).
 #define UMI_VARIANT_LIST(X) \
-    X(1, 8, 4)              \
-    X(1, 16, 4)             \
-    X(1, 26, 4)             \
-    X(1, 32, 3)             \
-    X(2, 32, 3)             \
-    X(4, 32, 3)             \
-    X(8, 24, 3)             \
-    X(8, 46, 2)             \
-    X(8, 46, 3)             \
-    X(16, 24, 4)            \
-    X(32, 12, 4)            \
-    X(16, 48, 2)            \
-    X(32, 48, 2)            \
-    X(32, 68, 2)            \
+    X(1, 8, 4)           \
+    X(1, 16, 4)          \
+    X(1, 26, 4)          \
+    X(1, 32, 3)          \
+    X(1, 40, 3)          \
+    X(1, 52, 2)          \
+    X(2, 32, 3)          \
+    X(2, 32, 2)          \
+    X(2, 38, 2)          \
+    X(2, 44, 2)          \
+    X(2, 52, 2)          \
+    X(2, 62, 2)          \
+    X(4, 32, 3)          \
+    X(4, 32, 2)          \
+    X(4, 38, 2)          \
+    X(4, 46, 2)          \
+    X(8, 24, 3)          \
+    X(4, 56, 2)          \
+    X(4, 68, 2)          \
+    X(8, 40, 2)          \
+    X(8, 46, 2)          \
+    X(8, 46, 3)          \
+    X(8, 48, 2)          \
+    X(16, 24, 4)         \
+    X(32, 12, 4)         \
+    X(8, 56, 2)          \
+    X(8, 68, 2)          \
+    X(16, 40, 2)         \
+    X(16, 48, 2)         \
+    X(16, 56, 2)         \
+    X(16, 68, 2)         \
+    X(32, 48, 2)         \
+    X(32, 56, 2)         \
+    X(32, 68, 2)         \
+    X(32, 92, 1)         \
+    X(32, 112, 1)        \
     X(32, 128, 1)
