@@ -230,10 +230,10 @@ void umi_default_segment_params(umi_segment_params *sp);
 /*
  * umi_detrend_batched with gap handling.  Same buffers and layout; `seg`
  * NULL means the defaults; `segments_out` (may be NULL) receives the number
- * of kept segments.  The segment scan needs the validity of every sample on
- * the host: the call enqueues a bit-packing kernel, copies 1 bit per sample
- * back and synchronises `stream` before it enqueues the batched launch (the
- * detrend itself stays asynchronous).  Scratch comes from cudaMallocAsync.
+ * of kept segments.  The scan counts each curve's segments on the device; the
+ * call copies the counts (16 bytes per curve) back and waits for them before
+ * it enqueues the batched launch (the detrend itself stays asynchronous).
+ * Scratch comes from cudaMallocAsync.
  */
 umi_status umi_detrend_segmented(const float *flux_d, const int64_t *offsets_h, const int32_t *W_h,
                                  int32_t B, const umi_params *params, const umi_segment_params *seg,

@@ -164,8 +164,8 @@ int persistent_grid(const Plan &plan, int flavour)
     return sms * per_sm;
 }
 
-static Curve make_curve(const float *flux, float *trend, float *detr, int64_t n, int W,
-                        const umi_params &p)
+Curve make_curve(const float *flux, float *trend, float *detr, int64_t n, int W,
+                 const umi_params &p)
 {
     Curve c;
     c.flux = flux;
@@ -313,15 +313,20 @@ umi_status BatchLayout::add_band(const Plan &plan, int flavour, const std::vecto
     return UMI_OK;
 }
 
-static Scratch scratch_layout(const BatchLayout &lay)
+Scratch scratch_layout(size_t n_curves, size_t n_bands)
 {
     Scratch s;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     s.curve_off = 0;
-    s.tile_off = up(lay.curves.size() * sizeof(Curve));
-    s.counter_off = s.tile_off + up(lay.curves.size() * sizeof(int32_t));
-    s.bytes = s.counter_off + up(std::max<size_t>(1, lay.bands.size()) * sizeof(uint32_t));
+    s.tile_off = up(n_curves * sizeof(Curve));
+    s.counter_off = s.tile_off + up(n_curves * sizeof(int32_t));
+    s.bytes = s.counter_off + up(std::max<size_t>(1, n_bands) * sizeof(uint32_t));
     return s;
+}
+
+static Scratch scratch_layout(const BatchLayout &lay)
+{
+    return scratch_layout(lay.curves.size(), lay.bands.size());
 }
 
 // Host image of the scratch: tables and zeroed counters.
@@ -332,8 +337,8 @@ static void write_tables(const BatchLayout &lay, const Scratch &sc, char *host)
     memset(host + sc.counter_off, 0, sc.bytes - sc.counter_off);
 }
 
-static umi_status enqueue_bands(const BatchLayout &lay, char *dev, const Scratch &sc,
-                                cudaStream_t stream, int *launches)
+umi_status enqueue_bands(const BatchLayout &lay, char *dev, const Scratch &sc, cudaStream_t stream,
+                         int *launches)
 {
     int nv = 0;
     const Variant *t = variant_table(&nv);
@@ -435,6 +440,19 @@ static void release_pinned(int slot, cudaStream_t stream)
         cudaStreamSynchronize(stream);
     }
 }
+
+umi_status PinnedStaging::acquire(size_t bytes) { return acquire_pinned(bytes, &slot, &p); }
+
+cudaError_t PinnedStaging::wait(cudaStream_t stream)
+{
+    cudaError_t e = cudaEventRecord(t_pinned[slot].ev, stream);
+    if (e == cudaSuccess) return cudaEventSynchronize(t_pinned[slot].ev);
+    // The event belongs to another device than this stream.
+    cudaGetLastError();
+    return cudaStreamSynchronize(stream);
+}
+
+void PinnedStaging::release(cudaStream_t stream) { release_pinned(slot, stream); }
 
 // The entry points take their device scratch with cudaMallocAsync from the
 // device's default memory pool.  Its release threshold is raised once per

@@ -151,6 +151,26 @@ struct Scratch {
     size_t curve_off = 0, tile_off = 0, counter_off = 0, bytes = 0;
 };
 
+Scratch scratch_layout(size_t n_curves, size_t n_bands);
+// Launches the bands of a layout whose tables lie at `dev`.
+umi_status enqueue_bands(const BatchLayout &lay, char *dev, const Scratch &sc, cudaStream_t stream,
+                         int *launches);
+
+Curve make_curve(const float *flux, float *trend, float *detr, int64_t n, int W, const umi_params &p);
+
+// A buffer of the calling thread's ring of pinned staging buffers.
+struct PinnedStaging {
+    char *p = nullptr;
+    umi_status acquire(size_t bytes);
+    // Waits for the work enqueued on `stream` so far.
+    cudaError_t wait(cudaStream_t stream);
+    // Lets the buffer be reused once the work enqueued on `stream` so far has run.
+    void release(cudaStream_t stream);
+
+private:
+    int slot = 0;
+};
+
 // A batch planned for caller-owned buffers: scratch.bytes of device memory and
 // as much (preferably pinned) host staging for the tables.
 struct PreparedBatch {
