@@ -265,6 +265,25 @@ __device__ __forceinline__ float select_rank(const float2 (&x)[R / 2], bool need
     float v;
     for (int p = 0;; ++p) {
         const bool more = __any_sync(0xffffffffu, need && lo < hi && clo != target && chi != target + 1);
+        if constexpr (ABS) {
+            if (!more) {
+                // Magnitudes are ordered as their bits are: the answer is the
+                // pattern nearest to lo from above, or to hi from below, both
+                // a smallest unsigned difference (the others wrap).
+                const bool up = clo == target;
+                const unsigned flip = up ? 0u : 0xffffffffu, add = up ? 0u - lo : hi + 1u;
+                unsigned r0 = 0xffffffffu, r1 = 0xffffffffu;
+#pragma unroll
+                for (int k = 0; k < R / 2; ++k) {
+                    r0 = __viaddmin_u32((__float_as_uint(x[k].x) & 0x7fffffffu) ^ flip, add, r0);
+                    r1 = __viaddmin_u32((__float_as_uint(x[k].y) & 0x7fffffffu) ^ flip, add, r1);
+                }
+                const unsigned r = group_umin<G>(min(r0, r1));
+                *below = up;
+                *le = chi;
+                return __uint_as_float(up ? lo + r : hi - r);
+            }
+        }
         if (!more || (p & 7) == kTighten) {
             // Smallest sample above lo - 1 and largest at or below hi.
             const float lof = ABS ? (lo ? sel_float<ABS>(lo - 1) : -1.f) : sel_float<ABS>(lo - 1);
@@ -582,7 +601,7 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
                 s = select_rank<G, R, true>(x, produce, 0u, __float_as_uint(0x1p98f), 0, st.nv,
                                             (st.nv - 1) >> 1, q0, __fdividef(q0, 0.43f * (float)st.nv), &le,
                                             &below);
-                mad = s;
+                mad = produce ? s : 0.f;
             }
             const bool iterate = produce && ((FLAGS & kFlagMad) != 0 ? (s > 0.f) : (msq > 0.f));
             if (__any_sync(0xffffffffu, iterate)) {
