@@ -17,6 +17,7 @@ from . import build as _build
 
 _lock = threading.Lock()
 _lib = None
+_torch = None
 
 UMI_OK = 0
 UMI_ERR_INVALID_ARG = 1
@@ -104,6 +105,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = False):
     """Load libumi.so (optionally building it first)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -208,36 +211,52 @@ def check_flags(clear=False) -> int:
     return int(f.value)
 
 
+def _t():
+    """torch, imported at the first call that takes tensors."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch
+
+
+# Addresses go to ctypes as plain integers (its c_void_p arguments take them):
+# a small curve's kernel runs for 6 us, so the binding's own microseconds are
+# most of such a call (one Kepler quarter 20.8 -> 13.7 us per call).
 def _stream_handle(stream):
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        # torch.cuda.current_stream() without the Stream object around it.
+        cuda = _t().cuda
+        return _torch._C._cuda_getCurrentRawStream(cuda.current_device())
+    return stream.cuda_stream
 
 
 def _dev_f32(t, name):
-    import torch
+    torch = _t()
     if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.float32 and t.is_contiguous()):
         raise TypeError("%s must be a contiguous float32 CUDA tensor" % name)
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def detrend(flux, W, p: Params | None = None, trend=None, detr=None, stream=None):
     """One curve on the GPU.  Returns (trend, detr) float32 CUDA tensors."""
-    import torch
     n = flux.numel()
-    trend = torch.empty_like(flux) if trend is None else trend
-    detr = torch.empty_like(flux) if detr is None else detr
-    _check_sizes(n, trend=trend, detr=detr)
-    _check(load().umi_detrend(_dev_f32(flux, "flux"), n, int(W), None if p is None else ctypes.byref(p),
-                              _dev_f32(trend, "trend"), _dev_f32(detr, "detr"), _stream_handle(stream)))
+    given = trend is not None or detr is not None
+    trend = _t().empty_like(flux) if trend is None else trend
+    detr = _t().empty_like(flux) if detr is None else detr
+    if given:
+        _check_sizes(n, trend=trend, detr=detr)
+    st = (_lib or load()).umi_detrend(_dev_f32(flux, "flux"), n, int(W), None if p is None else ctypes.byref(p),
+                                      _dev_f32(trend, "trend"), _dev_f32(detr, "detr"), _stream_handle(stream))
+    if st != UMI_OK:
+        _check(st)
     return trend, detr
 
 
 def detrend_diag(flux, W, p: Params | None = None, stream=None):
     """One curve with diagnostics.  Returns a dict of CUDA tensors:
     trend, detr, median, nvalid, nplus, scale."""
-    import torch
+    torch = _t()
     n = flux.numel()
     out = {"trend": torch.empty_like(flux), "detr": torch.empty_like(flux),
            "median": torch.empty_like(flux), "scale": torch.empty_like(flux),
@@ -281,7 +300,7 @@ def _csr_total(off):
 
 def detrend_batched(flux, offsets, W, p: Params | None = None, trend=None, detr=None, stream=None):
     """CSR batch on the GPU.  `offsets` [B+1] and `W` [B] are host arrays."""
-    import torch
+    torch = _t()
     off, offp = _host_i64(offsets)
     w, wp = _host_i32(W)
     B = off.size - 1
@@ -303,7 +322,7 @@ def detrend_batched_noalloc(flux, offsets, W, p: Params | None = None, trend=Non
     device memory for it (its work-queue tables go to a fixed 4 MiB device
     array), for callers that cannot allocate at this point.  Calls that
     overlap on the GPU share that array; keep them on one stream."""
-    import torch
+    torch = _t()
     off, offp = _host_i64(offsets)
     w, wp = _host_i32(W)
     B = off.size - 1
@@ -323,7 +342,7 @@ def detrend_segmented(flux, offsets, W, p: Params | None = None, gap_min=0, min_
                       detr=None, stream=None):
     """CSR batch with gap handling (umi_detrend_segmented).  Returns
     (trend, detr, kept_segments).  Synchronises the stream once (segment scan)."""
-    import torch
+    torch = _t()
     off, offp = _host_i64(offsets)
     w, wp = _host_i32(W)
     B = off.size - 1
