@@ -405,6 +405,131 @@ enum : int { kFlagDiag = 1, kFlagMad = 2 };
 // 4 bytes each.  The slice then holds T more floats after the staged samples.
 __host__ __device__ constexpr bool stages_outputs(int G) { return G <= 4; }
 
+// Two consecutive windows of a chain finish together in the 32-lane variants
+// of few slots: a lone window leaves the warp waiting for its reductions (ten
+// shuffles and a quotient per iteration against six slot pairs of work).
+// Together the two give the scheduler independent work, and their four sums
+// share one tree: each halving step keeps half of the sums per lane, so eight
+// shuffles serve both windows.  One curve of 18,000 samples at W = 361: 21.2 us,
+// 24.2 one window at a time.
+__host__ __device__ constexpr bool pairs_windows(int G, int R, int flags)
+{
+    return G == 32 && R <= 12 && (flags & kFlagMad) == 0;
+}
+
+// A window past Phase 1: its median, above-median count and output position.
+struct Pending {
+    float m;
+    float centre;
+    int gp;
+    int nv;
+    int64_t p;
+    bool produce;
+};
+
+// The 32-lane sum of a in lanes 0-15 and of b in lanes 16-31.
+__device__ __forceinline__ float half_sums(float a, float b, bool upper)
+{
+    float v = (upper ? b : a) + __shfl_xor_sync(0xffffffffu, upper ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Phases 2 and 3 of two windows whose residuals y = x - m are in ya and yb.
+// Lanes 0-15 own window a, lanes 16-31 window b.
+template <int R, int FLAGS>
+__device__ __forceinline__ void finish_pair(const Curve &cv, const Diag &dg, const float2 (&ya)[R / 2],
+                                            const float2 (&yb)[R / 2], const Pending &a, const Pending &b,
+                                            bool abs_form, float rho, float k1, int lane)
+{
+    const bool upper = (lane & 16) != 0;
+    const Pending own = upper ? b : a;
+    float mu = own.m, s = 0.f;
+    if (__any_sync(0xffffffffu, own.produce)) {
+        float2 sa = make_float2(0.f, 0.f), sb = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < R / 2; ++k) {
+            const float2 pa = make_float2(fmaxf(ya[k].x, 0.f), fmaxf(ya[k].y, 0.f));
+            const float2 pb = make_float2(fmaxf(yb[k].x, 0.f), fmaxf(yb[k].y, 0.f));
+            sa = __ffma2_rn(pa, pa, sa);
+            sb = __ffma2_rn(pb, pb, sb);
+        }
+        const float s2 = half_sums(sa.x + sa.y, sb.x + sb.y, upper);
+        const float msq = own.gp > 0 ? __fdividef(s2, (float)own.gp) : 0.f;
+        s = kScaleFactor * sqrtf(msq);  // for the diagnostic output
+        const bool iterate = own.produce && msq > 0.f;
+        if (__any_sync(0xffffffffu, iterate)) {
+            const float r = (msq >= 0x1p-126f) ? rsqrtf(msq) : 1.f / sqrtf(msq);
+            const float kp = r * k1, kp_o = __shfl_xor_sync(0xffffffffu, kp, 16);
+            const float ka = upper ? kp_o : kp, kb = upper ? kp : kp_o;
+            const float2 ka2 = make_float2(ka, ka), kb2 = make_float2(kb, kb);
+            const float na = cv.alpha * ka, nb = cv.alpha * kb;
+            const float2 na2 = make_float2(na, na), nb2 = make_float2(nb, nb);
+            const float2 rho2 = make_float2(rho, rho);
+            float delta = 0.f, da = 0.f, db = 0.f;
+#pragma unroll 1
+            for (int it = 0; it < cv.iters; ++it) {
+                float2 wa = make_float2(0.f, 0.f), wya = wa, wb = wa, wyb = wa;
+                // u_eff^2 as in the one-window form below.
+                auto slot = [&](const float2 y, float2 &w, float2 &wy, const float2 v, const float2 u) {
+                    const float2 z = make_float2(fma_sat(-u.x, v.x, 1.f), fma_sat(-u.y, v.y, 1.f));
+                    const float2 zz = __fmul2_rn(z, z);
+                    w = __fadd2_rn(w, zz);
+                    wy = __ffma2_rn(zz, y, wy);
+                };
+                if (abs_form) {
+                    const float2 ca = make_float2(-da * ka, -da * ka), cb = make_float2(-db * kb, -db * kb);
+#pragma unroll
+                    for (int k = 0; k < R / 2; ++k) {
+                        const float2 ta = __ffma2_rn(ya[k], ka2, ca), tb = __ffma2_rn(yb[k], kb2, cb);
+                        slot(ya[k], wa, wya, __ffma2_rn(rho2, make_float2(fabsf(ta.x), fabsf(ta.y)), ta), ta);
+                        slot(yb[k], wb, wyb, __ffma2_rn(rho2, make_float2(fabsf(tb.x), fabsf(tb.y)), tb), tb);
+                    }
+                } else {
+                    const float2 ca = make_float2(-da * ka, -da * ka), cb = make_float2(-db * kb, -db * kb);
+                    const float2 ea = make_float2(-da * na, -da * na), eb = make_float2(-db * nb, -db * nb);
+#pragma unroll
+                    for (int k = 0; k < R / 2; ++k) {
+                        const float2 pa = __ffma2_rn(ya[k], ka2, ca), qa = __ffma2_rn(ya[k], na2, ea);
+                        const float2 pb = __ffma2_rn(yb[k], kb2, cb), qb = __ffma2_rn(yb[k], nb2, eb);
+                        const float2 ua = make_float2(fminf(pa.x, qa.x), fminf(pa.y, qa.y));
+                        const float2 ub = make_float2(fminf(pb.x, qb.x), fminf(pb.y, qb.y));
+                        slot(ya[k], wa, wya, ua, ua);
+                        slot(yb[k], wb, wyb, ub, ub);
+                    }
+                }
+                // Lane bit 4 picks the window, bit 3 sum(w) or sum(w y).
+                const float fa = wa.x + wa.y, ga = wya.x + wya.y, fb = wb.x + wb.y, gb = wyb.x + wyb.y;
+                const float f = (upper ? fb : fa) + __shfl_xor_sync(0xffffffffu, upper ? fa : fb, 16);
+                const float g = (upper ? gb : ga) + __shfl_xor_sync(0xffffffffu, upper ? ga : gb, 16);
+                const bool second = (lane & 8) != 0;
+                float v = (second ? g : f) + __shfl_xor_sync(0xffffffffu, second ? f : g, 8);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                const float v_o = __shfl_xor_sync(0xffffffffu, v, 8);
+                const float sw = second ? v_o : v, swy = second ? v : v_o;
+                if (sw > 0.f) delta = __fdividef(swy, sw);
+                const float d_o = __shfl_xor_sync(0xffffffffu, delta, 16);
+                da = upper ? d_o : delta;
+                db = upper ? delta : d_o;
+            }
+            if (iterate) mu = own.m + delta;
+        }
+    }
+    if ((lane & 15) == 0 && own.p < cv.n) {
+        const float nanv = __int_as_float(0x7fc00000);
+        cv.trend[own.p] = own.produce ? mu : nanv;
+        cv.detr[own.p] = own.produce ? __fdiv_rn(own.centre, mu) : nanv;
+        if constexpr ((FLAGS & kFlagDiag) != 0) {
+            if (dg.median) dg.median[own.p] = (own.nv >= 1) ? own.m : nanv;
+            if (dg.nvalid) dg.nvalid[own.p] = own.nv;
+            if (dg.nplus) dg.nplus[own.p] = (own.nv >= 1) ? own.gp : 0;
+            if (dg.scale) dg.scale[own.p] = own.produce ? s : nanv;
+        }
+    }
+}
+
 template <int G, int R, int FLAGS>
 __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, const TileRef tile,
                                               float *out, int64_t t0, int q0, int P, int glane)
@@ -437,6 +562,8 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
     st.nv = 0;
     st.have = false;
     float mad = 0.f;  // the last window's MAD (kFlagMad)
+    float2 xh[pairs_windows(G, R, FLAGS) ? R / 2 : 1];  // the pair's first window
+    Pending held{};
 
 #pragma unroll 1
     for (int t = 0; t < P; ++t) {
@@ -566,6 +693,23 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
         const float centre = tile[q + h];
         const bool produce = (p < cv.n) && (st.nv >= 1) && (st.nv >= cv.min_valid) &&
                              (centre > kGapLimit);
+        if constexpr (pairs_windows(G, R, FLAGS)) {
+            const float2 neg = make_float2(-st.m, -st.m);
+#pragma unroll
+            for (int k = 0; k < R / 2; ++k) x[k] = __fadd2_rn(x[k], neg);
+            const Pending now{st.m, centre, st.Gp, st.nv, p, produce};
+            // An odd chain's last window has no partner.
+            const bool first = (t & 1) == 0;
+            if (first) {
+                held = now;
+#pragma unroll
+                for (int k = 0; k < R / 2; ++k) xh[k] = x[k];
+                if (t + 1 < P) continue;
+            }
+            const Pending none{0.f, 0.f, 0, 0, INT64_MAX, false};
+            finish_pair<R, FLAGS>(cv, dg, xh, x, held, first ? none : now, abs_form, rho, k1, glane);
+            continue;
+        }
         float mu = st.m;
         float s = 0.f;
         if (__any_sync(0xffffffffu, produce)) {
@@ -741,9 +885,10 @@ __device__ __forceinline__ int find_curve(const int32_t *__restrict__ first_tile
 // staged trend when stages_outputs(G).  MINB (CTAs of 256
 // threads per SM) sets the register budget the compiler aims for.  FLAGS
 // selects the diagnostic outputs and the MAD scale; every curve of one launch
-// must have the scale mode the kernel was built for.
+// must have the scale mode the kernel was built for.  Pairs of windows need 79
+// registers (at 64 they spill): 24 warps per SM.
 template <int G, int R, int MINB, int FLAGS>
-__global__ void __launch_bounds__(256, MINB) umi_tile_kernel(LaunchArgs a)
+__global__ void __launch_bounds__(256, pairs_windows(G, R, FLAGS) ? 3 : MINB) umi_tile_kernel(LaunchArgs a)
 {
     extern __shared__ float smem[];
     constexpr int S = G * R;

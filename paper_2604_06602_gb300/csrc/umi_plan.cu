@@ -241,9 +241,12 @@ void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
     int nv = 0;
     const Variant *t = variant_table(&nv);
     const int G = plan->G, groups = 32 / G;
-    const int64_t warps = (int64_t)std::max(1, device_info(current_device()).sms) * 8 * t[plan->variant].minb;
-    const int64_t steps = (positions + warps * groups - 1) / (warps * groups);
+    const bool pairs = pairs_windows(G, plan->R, 0);
+    const int64_t warps =
+        (int64_t)std::max(1, device_info(current_device()).sms) * 8 * (pairs ? 3 : t[plan->variant].minb);
+    int64_t steps = (positions + warps * groups - 1) / (warps * groups);
     if (steps <= G) {
+        if (pairs) steps += steps & 1;  // windows are worked on two at a time
         plan->chain = (int)std::max<int64_t>(1, steps);
         return;
     }
