@@ -565,13 +565,15 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
     float2 xh[pairs_windows(G, R, FLAGS) ? R / 2 : 1];  // the pair's first window
     Pending held{};
 
+    int q = q0 - 1, left = P;
+    bool begin = true;
 #pragma unroll 1
-    for (int t = 0; t < P; ++t) {
-        const int q = q0 + t;
+    for (; left > 0; --left) {
+        ++q;
         const int64_t p = t0 + q;
 
         // ---- slide: one sample leaves, one enters --------------------------
-        if (t > 0) {
+        if (!begin) {
             const float out = tile[q - 1];
             const float in = tile[q + W - 1];
             const bool ov = out > kGapLimit;
@@ -593,7 +595,8 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
 
         load_window<G, R>(x, tile, q, glane, W, tail_only);
 
-        if (t == 0) {
+        if (begin) {
+            begin = false;
             int c = 0;
 #pragma unroll
             for (int k = 0; k < R / 2; ++k)
@@ -699,12 +702,12 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
             for (int k = 0; k < R / 2; ++k) x[k] = __fadd2_rn(x[k], neg);
             const Pending now{st.m, centre, st.Gp, st.nv, p, produce};
             // An odd chain's last window has no partner.
-            const bool first = (t & 1) == 0;
+            const bool first = ((P - left) & 1) == 0;
             if (first) {
                 held = now;
 #pragma unroll
                 for (int k = 0; k < R / 2; ++k) xh[k] = x[k];
-                if (t + 1 < P) continue;
+                if (left > 1) continue;
             }
             const Pending none{0.f, 0.f, 0, 0, INT64_MAX, false};
             finish_pair<R, FLAGS>(cv, dg, xh, x, held, first ? none : now, abs_form, rho, k1, glane);
