@@ -895,6 +895,9 @@ __global__ void __launch_bounds__(256, pairs_windows(G, R, FLAGS) ? 3 : MINB) um
 {
     extern __shared__ float smem[];
     constexpr int S = G * R;
+    // Launched as a programmatic dependent (see the launcher): nothing of
+    // global memory is touched before the work ahead in the stream is done.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int n_warps = blockDim.x >> 5;
