@@ -222,7 +222,7 @@ umi_status launch_single_curve(const Curve &c, int64_t plan_positions, const Dia
     Plan plan;
     umi_status st = single_plan(c.W, plan_positions, c.n, &plan);
     if (st != UMI_OK) return st;
-    const int flavour = (diag ? kFlagDiag : 0) | (c.scale_mode == UMI_SCALE_MAD ? kFlagMad : 0);
+    const int flavour = (diag ? kFlagDiag : 0) | curve_flavour(c);
     st = prepare_kernel(plan, flavour);
     if (st != UMI_OK) return st;
     const int64_t T = plan.tile();
@@ -296,7 +296,7 @@ umi_status build_layout(const std::vector<Curve> &curves, BatchLayout *layout,
             it = plans.emplace(key, p).first;
         }
         const Plan &p = it->second;
-        const int flavour = curves[b].scale_mode == UMI_SCALE_MAD ? kFlagMad : 0;
+        const int flavour = curve_flavour(curves[b]);
         // Untuned plans of one variant share a launch, whose chain is fitted below.
         by_plan[std::make_tuple(-p.G * p.R, p.variant, p.tuned ? p.chain : 0, p.threads, flavour)]
             .push_back((int)b);

@@ -80,7 +80,7 @@ uint64_t tune_epoch();
 void plan_out(const Plan &p, umi_plan *out);
 umi_status check_params(const umi_params *p, umi_params *out);
 int resolve_min_valid(int W, int min_valid);
-// `flavour` = kFlagDiag | kFlagMad bits (the kernel build to use).
+// `flavour` = kFlagDiag, kFlagMad and kFlagMin bits (the kernel build to use).
 umi_status prepare_kernel(const Plan &plan, int flavour);
 // Persistent grid size for a plan on the current device.
 int persistent_grid(const Plan &plan, int flavour);
@@ -131,7 +131,7 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
 struct BatchLayout {
     struct Band {
         Plan plan;
-        int flavour = 0;  // kFlagMad when the band's curves use the MAD scale
+        int flavour = 0;  // curve_flavour of the band's curves
         int32_t first_curve = 0;
         int32_t n_curves = 0;
         int32_t n_items = 0;

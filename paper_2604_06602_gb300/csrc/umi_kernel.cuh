@@ -350,6 +350,39 @@ __device__ __forceinline__ float select_rank(const float2 (&x)[R / 2], bool need
     return v;
 }
 
+// a b + c per component, as one packed instruction or two scalar ones (the
+// same values either way).
+template <bool SCALAR>
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    return SCALAR ? make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)) : __ffma2_rn(a, b, c);
+}
+
+// Which of the iteration's FMAs are scalar pairs.  The FMA pipe takes two
+// cycles for a packed instruction and one for a scalar one, so the mixes cost
+// the same there, but some are scheduled better.  Each lane split has the mix
+// that its variants like best of 32 (kernel times, all packed against it: W = 25
+// (1,26) 0.576 -> 0.569 ms, W = 49 (1,52) 0.566 -> 0.550, W = 73 (2,38) 0.647 ->
+// 0.633, W = 361 (8,46) 2.595 -> 2.515, W = 541 (8,68) 1.839 -> 1.829, W = 721
+// (16,48) 1.807 -> 1.795, W = 1441 (32,48) 1.916 -> 1.893; W = 217 (4,56) has
+// none that is better for (4,46) too).  The min form's second residual is
+// scalar everywhere (alpha = 10: W = 361 2.851 -> 2.759 ms, W = 73 0.713 -> 0.684,
+// W = 2161 5.444 -> 5.404).
+struct IterationForm {
+    bool t;    // t = sigma (y - delta)
+    bool v;    // t + rho |t|
+    bool swy;  // sum w y
+};
+__host__ __device__ constexpr IterationForm iteration_form(int G, int R)
+{
+    return G == 1    ? IterationForm{true, false, true}
+           : G == 2  ? IterationForm{true, true, true}
+           : G == 8  ? IterationForm{false, false, true}
+           : G == 16 ? IterationForm{R <= 48, false, false}
+           : G == 32 ? IterationForm{true, false, true}
+                     : IterationForm{false, false, false};
+}
+
 // Load the window of tile position q into registers: slot s = glane + G*i
 // holds tile[q + s] for s < W, kGap past W.  Slots are stored in pairs
 // (i = 2k, 2k+1 in x[k].x, x[k].y) for the packed FP32x2 arithmetic.
@@ -395,8 +428,20 @@ struct MedianState {
     bool have;
 };
 
-// Kernel flags: diagnostic outputs, MAD scale instead of Eq. 1.
-enum : int { kFlagDiag = 1, kFlagMad = 2 };
+// Kernel flags: diagnostic outputs, MAD scale instead of Eq. 1, the min form of
+// Eq. 2's sign select (uses_min_form).  Each form has kernels of its own: with
+// both in one kernel the schedule of either loop moved by up to 4 % with the
+// other's.
+enum : int { kFlagDiag = 1, kFlagMad = 2, kFlagMin = 4 };
+
+// The |t| form of the sign select serves 1/4 <= alpha <= 4 (process_chain).
+__host__ __device__ inline bool uses_min_form(float alpha) { return !(alpha >= 0.25f && alpha <= 4.f); }
+
+// The kernel build a curve needs (without kFlagDiag).
+__host__ __device__ inline int curve_flavour(const Curve &c)
+{
+    return (c.scale_mode != 0 ? kFlagMad : 0) | (uses_min_form(c.alpha) ? kFlagMin : 0);
+}
 
 // Narrow groups (G <= 4 lanes per window) stage their trend values in the
 // warp's shared-memory slice and write trend and detrended flux at the end of
@@ -441,8 +486,9 @@ __device__ __forceinline__ float half_sums(float a, float b, bool upper)
 template <int R, int FLAGS>
 __device__ __forceinline__ void finish_pair(const Curve &cv, const Diag &dg, const float2 (&ya)[R / 2],
                                             const float2 (&yb)[R / 2], const Pending &a, const Pending &b,
-                                            bool abs_form, float rho, float k1, int lane)
+                                            float rho, float k1, int lane)
 {
+    constexpr bool abs_form = (FLAGS & kFlagMin) == 0;
     const bool upper = (lane & 16) != 0;
     const Pending own = upper ? b : a;
     float mu = own.m, s = 0.f;
@@ -478,7 +524,7 @@ __device__ __forceinline__ void finish_pair(const Curve &cv, const Diag &dg, con
                     w = __fadd2_rn(w, zz);
                     wy = __ffma2_rn(zz, y, wy);
                 };
-                if (abs_form) {
+                if constexpr (abs_form) {
                     const float2 ca = make_float2(-da * ka, -da * ka), cb = make_float2(-db * kb, -db * kb);
 #pragma unroll
                     for (int k = 0; k < R / 2; ++k) {
@@ -548,7 +594,7 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
     // relative at a = 4); every other alpha takes the min of two scaled
     // residuals.  With r = 1/sqrt(msq) (Phase 2), sigma = r k1 in that form,
     // and in the other kp = r k1, kn = alpha kp (k1 negated when alpha < 1).
-    const bool abs_form = alpha >= 0.25f && alpha <= 4.f;
+    constexpr bool abs_form = (FLAGS & kFlagMin) == 0;
     const float rho = fmaf(-alpha, alpha, 1.f) / fmaf(alpha, alpha, 1.f);
     const float k1 = (abs_form ? sqrtf(0.5f * fmaf(alpha, alpha, 1.f)) : (alpha >= 1.f ? 1.f : -1.f)) /
                      (kScaleFactor * cst);
@@ -710,7 +756,7 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
                 if (left > 1) continue;
             }
             const Pending none{0.f, 0.f, 0, 0, INT64_MAX, false};
-            finish_pair<R, FLAGS>(cv, dg, xh, x, held, first ? none : now, abs_form, rho, k1, glane);
+            finish_pair<R, FLAGS>(cv, dg, xh, x, held, first ? none : now, rho, k1, glane);
             continue;
         }
         float mu = st.m;
@@ -760,7 +806,7 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
                 if constexpr ((FLAGS & kFlagMad) != 0) r = kScaleFactor / s;
                 else r = (msq >= 0x1p-126f) ? rsqrtf(msq) : 1.f / sqrtf(msq);
                 float delta = 0.f;
-                if (abs_form) {
+                if constexpr (abs_form) {
                     // t = sigma (y - delta), sigma^2 = (kp^2 + kn^2)/2:
                     // t (t + rho |t|) = kp^2 u^2 for u >= 0, kn^2 u^2 for u < 0,
                     // so one FMA with |t| as an operand does the sign select.
@@ -773,33 +819,13 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
                         float2 swt = make_float2(0.f, 0.f), swyt = make_float2(0.f, 0.f);
 #pragma unroll
                         for (int k = 0; k < R / 2; ++k) {
-                            const float2 ts = __ffma2_rn(x[k], sg2, c0);
-                            // t + rho |t| per slot: one FFMA2 with |t| as its
-                            // operand, or two scalar FMAs (the same value
-                            // either way); the scalar pair schedules better
-                            // in the 8-lane variants (0.25 % on 1000 TESS
-                            // curves), the packed form in the others (3.3 % on
-                            // the 32-lane W = 2161 batch).
-                            float2 v;
-                            if constexpr (G != 8) {
-                                v = __ffma2_rn(rho2, make_float2(fabsf(ts.x), fabsf(ts.y)), ts);
-                            } else {
-                                v = make_float2(fmaf(rho, fabsf(ts.x), ts.x), fmaf(rho, fabsf(ts.y), ts.y));
-                            }
+                            constexpr IterationForm form = iteration_form(G, R);
+                            const float2 ts = fma2<form.t>(x[k], sg2, c0);
+                            const float2 v = fma2<form.v>(rho2, make_float2(fabsf(ts.x), fabsf(ts.y)), ts);
                             const float2 z = make_float2(fma_sat(-ts.x, v.x, 1.f), fma_sat(-ts.y, v.y, 1.f));
-                            if constexpr (G == 1) {
-                                // sum z^2 and sum z (z y): the same three
-                                // packed instructions, scheduled 1.6 % faster
-                                // in the one-lane variants (the W = 25 band)
-                                // and 1 % slower in the others.
-                                const float2 zy = __fmul2_rn(z, x[k]);
-                                swt = __ffma2_rn(z, z, swt);
-                                swyt = __ffma2_rn(z, zy, swyt);
-                            } else {
-                                const float2 w = __fmul2_rn(z, z);
-                                swt = __fadd2_rn(swt, w);
-                                swyt = __ffma2_rn(w, x[k], swyt);
-                            }
+                            const float2 w = __fmul2_rn(z, z);
+                            swt = __fadd2_rn(swt, w);
+                            swyt = fma2<form.swy>(w, x[k], swyt);
                         }
                         const float sws = group_sum<G>(swt.x + swt.y);
                         const float swys = group_sum<G>(swyt.x + swyt.y);
@@ -823,7 +849,7 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
 #pragma unroll
                         for (int k = 0; k < R / 2; ++k) {
                             const float2 p1 = __ffma2_rn(x[k], kp2, c1);
-                            const float2 p2 = __ffma2_rn(x[k], kn2, c2);
+                            const float2 p2 = fma2<true>(x[k], kn2, c2);
                             const float qa = fminf(p1.x, p2.x);
                             const float qb = fminf(p1.y, p2.y);
                             const float2 z = make_float2(fma_sat(-qa, qa, 1.f), fma_sat(-qb, qb, 1.f));
@@ -887,8 +913,9 @@ __device__ __forceinline__ int find_curve(const int32_t *__restrict__ first_tile
 // Dynamic shared memory: warps * (T + S - 1) floats, plus warps * T for the
 // staged trend when stages_outputs(G).  MINB (CTAs of 256
 // threads per SM) sets the register budget the compiler aims for.  FLAGS
-// selects the diagnostic outputs and the MAD scale; every curve of one launch
-// must have the scale mode the kernel was built for.  Pairs of windows need 79
+// selects the diagnostic outputs, the MAD scale and the sign select's form;
+// every curve of one launch must have the scale mode and an alpha that the
+// kernel was built for (curve_flavour).  Pairs of windows need 79
 // registers (at 64 they spill): 24 warps per SM.
 template <int G, int R, int MINB, int FLAGS>
 __global__ void __launch_bounds__(256, pairs_windows(G, R, FLAGS) ? 3 : MINB) umi_tile_kernel(LaunchArgs a)

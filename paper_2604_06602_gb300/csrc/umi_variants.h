@@ -12,8 +12,8 @@ namespace umi {
 typedef cudaError_t (*LaunchFn)(const LaunchArgs &args, int grid, int threads, size_t smem,
                                 cudaStream_t stream);
 
-// Kernel flavours: index = kFlagDiag | kFlagMad bits.
-constexpr int kFlavours = 4;
+// Kernel flavours: index = kFlagDiag | kFlagMad | kFlagMin bits.
+constexpr int kFlavours = 8;
 
 struct Variant {
     int G;
@@ -63,19 +63,25 @@ const Variant *variant_table(int *count);
     {                                                                                         \
         return launch_dependent(umi_tile_kernel<G_, R_, M_, F>, a, grid, threads, smem, st);  \
     }                                                                                         \
+    template <int F>                                                                          \
+    static void UMI_VNAME(fill_flavour_, G_, R_, M_)(Variant * v)                             \
+    {                                                                                         \
+        v->launch[F] = UMI_VNAME(launch_, G_, R_, M_)<F>;                                     \
+        v->kernel[F] = (const void *)umi_tile_kernel<G_, R_, M_, F>;                          \
+    }                                                                                         \
     void UMI_VNAME(fill_, G_, R_, M_)(Variant * v)                                            \
     {                                                                                         \
         v->G = G_;                                                                            \
         v->R = R_;                                                                            \
         v->minb = M_;                                                                         \
-        v->launch[0] = UMI_VNAME(launch_, G_, R_, M_)<0>;                                     \
-        v->launch[1] = UMI_VNAME(launch_, G_, R_, M_)<1>;                                     \
-        v->launch[2] = UMI_VNAME(launch_, G_, R_, M_)<2>;                                     \
-        v->launch[3] = UMI_VNAME(launch_, G_, R_, M_)<3>;                                     \
-        v->kernel[0] = (const void *)umi_tile_kernel<G_, R_, M_, 0>;                          \
-        v->kernel[1] = (const void *)umi_tile_kernel<G_, R_, M_, 1>;                          \
-        v->kernel[2] = (const void *)umi_tile_kernel<G_, R_, M_, 2>;                          \
-        v->kernel[3] = (const void *)umi_tile_kernel<G_, R_, M_, 3>;                          \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<0>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<1>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<2>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<3>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<4>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<5>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<6>(v);                                           \
+        UMI_VNAME(fill_flavour_, G_, R_, M_)<7>(v);                                           \
     }                                                                                         \
     }
 
