@@ -46,8 +46,8 @@ LANES_PER_SM = 128
 # headline workload, from the ncu capture of that workload, valid only while
 # the kernel's code (comments and blank lines removed) hashes to
 # `kernel_sha256`.
-MEASURED_TRAFFIC = {"bytes": 163.02e6,
-                    "kernel_sha256": "006aa279044fa5dccee93fc0fde15514b0bfb5f854327c42d3daa2726affd0c7"}
+MEASURED_TRAFFIC = {"bytes": 161.03e6,
+                    "kernel_sha256": "2e39b8cad13b8210945b297d7cca6d7487c39cda42167bac5b14db3691fe510e"}
 KERNEL_SOURCE = os.path.join(ROOT, "paper_2604_06602_gb300", "csrc", "umi_kernel.cuh")
 
 
