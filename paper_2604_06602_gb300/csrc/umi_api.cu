@@ -478,14 +478,16 @@ static void release_pinned(int slot, cudaStream_t stream)
 
 umi_status PinnedStaging::acquire(size_t bytes) { return acquire_pinned(bytes, &slot, &p); }
 
-cudaError_t PinnedStaging::wait(cudaStream_t stream)
+cudaError_t PinnedStaging::mark(cudaStream_t stream)
 {
-    cudaError_t e = cudaEventRecord(t_pinned[slot].ev, stream);
-    if (e == cudaSuccess) return cudaEventSynchronize(t_pinned[slot].ev);
+    marked = cudaEventRecord(t_pinned[slot].ev, stream) == cudaSuccess;
+    if (marked) return cudaSuccess;
     // The event belongs to another device than this stream.
     cudaGetLastError();
     return cudaStreamSynchronize(stream);
 }
+
+cudaError_t PinnedStaging::wait() { return marked ? cudaEventSynchronize(t_pinned[slot].ev) : cudaSuccess; }
 
 void PinnedStaging::release(cudaStream_t stream) { release_pinned(slot, stream); }
 

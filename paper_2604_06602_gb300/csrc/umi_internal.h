@@ -162,13 +162,15 @@ Curve make_curve(const float *flux, float *trend, float *detr, int64_t n, int W,
 struct PinnedStaging {
     char *p = nullptr;
     umi_status acquire(size_t bytes);
-    // Waits for the work enqueued on `stream` so far.
-    cudaError_t wait(cudaStream_t stream);
+    // Marks the work enqueued on `stream` so far, and waits for it.
+    cudaError_t mark(cudaStream_t stream);
+    cudaError_t wait();
     // Lets the buffer be reused once the work enqueued on `stream` so far has run.
     void release(cudaStream_t stream);
 
 private:
     int slot = 0;
+    bool marked = false;
 };
 
 // A batch planned for caller-owned buffers: scratch.bytes of device memory and

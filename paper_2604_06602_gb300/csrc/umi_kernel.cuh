@@ -265,24 +265,26 @@ __device__ __forceinline__ float select_rank(const float2 (&x)[R / 2], bool need
     float v;
     for (int p = 0;; ++p) {
         const bool more = __any_sync(0xffffffffu, need && lo < hi && clo != target && chi != target + 1);
-        if constexpr (ABS) {
-            if (!more) {
-                // Magnitudes are ordered as their bits are: the answer is the
-                // pattern nearest to lo from above, or to hi from below, both
-                // a smallest unsigned difference (the others wrap).
-                const bool up = clo == target;
-                const unsigned flip = up ? 0u : 0xffffffffu, add = up ? 0u - lo : hi + 1u;
-                unsigned r0 = 0xffffffffu, r1 = 0xffffffffu;
+        if (!more && (ABS || __all_sync(0xffffffffu, !need || lo > 0x80000000u))) {
+            // Magnitudes, and samples above zero, are ordered as their bits
+            // are: the answer is the pattern nearest to lo from above, or to hi
+            // from below, both a smallest unsigned difference (the other
+            // patterns, negative samples among them, are further away or
+            // wrap).
+            const bool up = clo == target;
+            const unsigned lob = lo & 0x7fffffffu, hib = hi & 0x7fffffffu;
+            const unsigned flip = up ? 0u : 0xffffffffu, add = up ? 0u - lob : hib + 1u;
+            unsigned r0 = 0xffffffffu, r1 = 0xffffffffu;
 #pragma unroll
-                for (int k = 0; k < R / 2; ++k) {
-                    r0 = __viaddmin_u32((__float_as_uint(x[k].x) & 0x7fffffffu) ^ flip, add, r0);
-                    r1 = __viaddmin_u32((__float_as_uint(x[k].y) & 0x7fffffffu) ^ flip, add, r1);
-                }
-                const unsigned r = group_umin<G>(min(r0, r1));
-                *below = up;
-                *le = chi;
-                return __uint_as_float(up ? lo + r : hi - r);
+            for (int k = 0; k < R / 2; ++k) {
+                const unsigned a = __float_as_uint(x[k].x), b = __float_as_uint(x[k].y);
+                r0 = __viaddmin_u32((ABS ? a & 0x7fffffffu : a) ^ flip, add, r0);
+                r1 = __viaddmin_u32((ABS ? b & 0x7fffffffu : b) ^ flip, add, r1);
             }
+            const unsigned r = group_umin<G>(min(r0, r1));
+            *below = up;
+            *le = chi;
+            return __uint_as_float(up ? lob + r : hib - r);
         }
         if (!more || (p & 7) == kTighten) {
             // Smallest sample above lo - 1 and largest at or below hi.
@@ -376,7 +378,7 @@ struct IterationForm {
 __host__ __device__ constexpr IterationForm iteration_form(int G, int R)
 {
     return G == 1    ? IterationForm{true, false, true}
-           : G == 2  ? IterationForm{true, true, true}
+           : G == 2  ? IterationForm{R <= 38, R <= 38, true}
            : G == 8  ? IterationForm{false, false, true}
            : G == 16 ? IterationForm{R <= 48, false, false}
            : G == 32 ? IterationForm{true, false, true}
@@ -679,11 +681,11 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
             const float mf = select_rank<G, R, false>(
                 x, need_full, mn == 0.f ? 0x7fffffffu : float_key(mn), mx == 0.f ? 0x80000000u : float_key(mx),
                 S - st.nv, S, (S - st.nv) + k, 0.f, 0.f, &le, &below);
-            int ce = 0;
+            float2 ef = make_float2(0.f, 0.f);  // 0/1 flags, exact below 2^24
 #pragma unroll
             for (int k2 = 0; k2 < R / 2; ++k2)
-                ce += ((x[k2].x == mf) ? 1 : 0) + ((x[k2].y == mf) ? 1 : 0);
-            ce = group_sum_int<G>(ce);
+                ef = __fadd2_rn(ef, make_float2(eq_flag(x[k2].x, mf), eq_flag(x[k2].y, mf)));
+            const int ce = group_sum_int<G>((int)(ef.x + ef.y));
             if (need_full) {
                 st.m = mf;
                 st.L = below ? k : le - ce - (S - st.nv);

@@ -330,10 +330,12 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
     }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(stage.p + count_off, d_counts, C * sizeof(SegmentCount), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = stage.wait(stream);
-    // NaN everywhere; kept segments are overwritten by the batch below.
+    if (e == cudaSuccess) e = stage.mark(stream);
+    // NaN everywhere while the host waits for the counts; kept segments are
+    // overwritten by the batch below.
     if (e == cudaSuccess) e = cudaMemsetAsync(trend, 0xff, sizeof(float) * (size_t)total, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(detr, 0xff, sizeof(float) * (size_t)total, stream);
+    if (e == cudaSuccess) e = stage.wait();
     if (e != cudaSuccess) {
         stage.release(stream);
         cudaFreeAsync(scan, stream);
