@@ -62,6 +62,10 @@ class ArenaAllocator {
     std::map<size_t, size_t> free_;  // offset -> length
 };
 
+// The gap split's rule in sequential form, over the validity mask: the model of
+// the device scan (umi_segments.cu), which the host tests hold against a scan
+// by samples.
+//
 // Reader over the 32-bit-word validity mask: word-at-a-time run scans.
 struct Bits {
     const unsigned *w;

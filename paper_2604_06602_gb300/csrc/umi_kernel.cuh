@@ -365,11 +365,12 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
 // the same there, but some are scheduled better.  Each lane split has the mix
 // that its variants like best of 32 (kernel times, all packed against it: W = 25
 // (1,26) 0.576 -> 0.569 ms, W = 49 (1,52) 0.566 -> 0.550, W = 73 (2,38) 0.647 ->
-// 0.633, W = 361 (8,46) 2.595 -> 2.515, W = 541 (8,68) 1.839 -> 1.829, W = 721
-// (16,48) 1.807 -> 1.795, W = 1441 (32,48) 1.916 -> 1.893; W = 217 (4,56) has
-// none that is better for (4,46) too).  The min form's second residual is
-// scalar everywhere (alpha = 10: W = 361 2.851 -> 2.759 ms, W = 73 0.713 -> 0.684,
-// W = 2161 5.444 -> 5.404).
+// 0.633, W = 97 (2,52) 0.662 -> 0.647, W = 217 (4,56) 1.342 -> 1.329, W = 361
+// (8,46) 2.595 -> 2.515, W = 541 (8,68) 1.839 -> 1.829, W = 721 (16,48) 1.807 ->
+// 1.795, W = 1441 (32,48) 1.916 -> 1.894, W = 2161 (32,68) 9.41 -> 9.39; (4,46),
+// (16,56) and (16,68) have none that is better).  The min form's second
+// residual is scalar everywhere (alpha = 10: W = 361 2.851 -> 2.759 ms, W = 73
+// 0.713 -> 0.684, W = 2161 5.444 -> 5.404).
 struct IterationForm {
     bool t;    // t = sigma (y - delta)
     bool v;    // t + rho |t|
@@ -379,10 +380,10 @@ __host__ __device__ constexpr IterationForm iteration_form(int G, int R)
 {
     return G == 1    ? IterationForm{true, false, true}
            : G == 2  ? IterationForm{R <= 38, R <= 38, true}
+           : G == 4  ? IterationForm{false, false, R >= 56}
            : G == 8  ? IterationForm{false, false, true}
            : G == 16 ? IterationForm{R <= 48, false, false}
-           : G == 32 ? IterationForm{true, false, true}
-                     : IterationForm{false, false, false};
+                     : IterationForm{R <= 48, false, true};
 }
 
 // Load the window of tile position q into registers: slot s = glane + G*i

@@ -22,7 +22,6 @@
 #include <string>
 #include <vector>
 
-#include "umi_host.h"
 #include "umi_internal.h"
 
 namespace umi {
