@@ -46,8 +46,8 @@ LANES_PER_SM = 128
 # headline workload, from the ncu capture of that workload, valid only while
 # the kernel's code (comments and blank lines removed) hashes to
 # `kernel_sha256`.
-MEASURED_TRAFFIC = {"bytes": 161.03e6,
-                    "kernel_sha256": "2e39b8cad13b8210945b297d7cca6d7487c39cda42167bac5b14db3691fe510e"}
+MEASURED_TRAFFIC = {"bytes": 160.99e6,
+                    "kernel_sha256": "b12d477e2414ad0848de8435d782ebd45adfbb3021171a98867757779c25c7a5"}
 KERNEL_SOURCE = os.path.join(ROOT, "paper_2604_06602_gb300", "csrc", "umi_kernel.cuh")
 
 
