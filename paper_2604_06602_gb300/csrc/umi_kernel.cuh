@@ -256,7 +256,8 @@ __device__ __forceinline__ float sel_float(unsigned k)
 // so no input takes more than twice the key width.  One TESS curve (a select
 // every 8 windows) 26.2 -> 25.1 us.  `q`, `dq`: first pivot
 // and the spacing of one rank there (dq > 0), for the first three pivots.
-template <int G, int R, bool ABS>
+// BITS: positive samples may be picked by their bit patterns.
+template <int G, int R, bool ABS, bool BITS = true>
 __device__ __forceinline__ float select_rank(const float2 (&x)[R / 2], bool need, unsigned lo, unsigned hi,
                                              int clo, int chi, int target, float q, float dq, int *le,
                                              bool *below)
@@ -265,7 +266,7 @@ __device__ __forceinline__ float select_rank(const float2 (&x)[R / 2], bool need
     float v;
     for (int p = 0;; ++p) {
         const bool more = __any_sync(0xffffffffu, need && lo < hi && clo != target && chi != target + 1);
-        if (!more && (ABS || __all_sync(0xffffffffu, !need || lo > 0x80000000u))) {
+        if (!more && (ABS || (BITS && __all_sync(0xffffffffu, !need || lo > 0x80000000u)))) {
             // Magnitudes, and samples above zero, are ordered as their bits
             // are: the answer is the pattern nearest to lo from above, or to hi
             // from below, both a smallest unsigned difference (the other
@@ -386,6 +387,22 @@ __host__ __device__ constexpr IterationForm iteration_form(int G, int R)
                      : IterationForm{R <= 48, false, true};
 }
 
+// Kernel flags: diagnostic outputs, MAD scale instead of Eq. 1, the min form of
+// Eq. 2's sign select (uses_min_form).  Each form has kernels of its own: with
+// both in one kernel the schedule of either loop moved by up to 4 % with the
+// other's.
+enum : int { kFlagDiag = 1, kFlagMad = 2, kFlagMin = 4 };
+
+// Whether a select may pick a positive sample by its bit patterns
+// (select_rank).  That pass is the shorter one, but the min form's loops of 8
+// lanes up to 46 slots and of long 2-lane windows are scheduled better without
+// it (alpha = 10, 300 curves at W = 361: 2.781 -> 2.729 ms; 495 curves at
+// W = 121: 1.568 -> 1.533 ms); its other variants lose 0.1 to 1 % without it.
+__host__ __device__ constexpr bool picks_by_bits(int G, int R, int flags)
+{
+    return (flags & kFlagMin) == 0 || !((G == 8 && R <= 46) || (G == 2 && R > 38));
+}
+
 // Load the window of tile position q into registers: slot s = glane + G*i
 // holds tile[q + s] for s < W, kGap past W.  Slots are stored in pairs
 // (i = 2k, 2k+1 in x[k].x, x[k].y) for the packed FP32x2 arithmetic.
@@ -430,12 +447,6 @@ struct MedianState {
     int nv;    // valid samples in the window
     bool have;
 };
-
-// Kernel flags: diagnostic outputs, MAD scale instead of Eq. 1, the min form of
-// Eq. 2's sign select (uses_min_form).  Each form has kernels of its own: with
-// both in one kernel the schedule of either loop moved by up to 4 % with the
-// other's.
-enum : int { kFlagDiag = 1, kFlagMad = 2, kFlagMin = 4 };
 
 // The |t| form of the sign select serves 1/4 <= alpha <= 4 (process_chain).
 __host__ __device__ inline bool uses_min_form(float alpha) { return !(alpha >= 0.25f && alpha <= 4.f); }
@@ -679,7 +690,7 @@ __device__ __forceinline__ void process_chain(const Curve &cv, const Diag &dg, c
             mx = group_max<G>(mx);
             int le;
             bool below;
-            const float mf = select_rank<G, R, false>(
+            const float mf = select_rank<G, R, false, picks_by_bits(G, R, FLAGS)>(
                 x, need_full, mn == 0.f ? 0x7fffffffu : float_key(mn), mx == 0.f ? 0x80000000u : float_key(mx),
                 S - st.nv, S, (S - st.nv) + k, 0.f, 0.f, &le, &below);
             float2 ef = make_float2(0.f, 0.f);  // 0/1 flags, exact below 2^24
