@@ -94,8 +94,6 @@ umi_status check_params(const umi_params *p, umi_params *out)
     return UMI_OK;
 }
 
-static std::mutex g_attr_mu;
-
 // ---------------------------------------------------------- checked build --
 // Builds compiled with UMI_CHECKED give every launch a device flag word (one
 // per device, allocated by prepare_kernel, which runs before any launch or
@@ -139,11 +137,14 @@ umi_status prepare_kernel(const Plan &plan, int flavour)
     }
     const size_t smem = plan.smem_bytes();
     if (smem > 48 * 1024) {
-        if (smem > device_info(current_device()).smem_optin)
+        // The limit belongs to the kernel, not to this launch: it is always set to
+        // the device's, so that neither another band of this call nor another
+        // thread lowers it between here and the launch.
+        const size_t limit = device_info(current_device()).smem_optin;
+        if (smem > limit)
             return fail(UMI_ERR_INVALID_ARG, "tile needs more shared memory than the device allows");
-        std::lock_guard<std::mutex> lk(g_attr_mu);
         const void *k = t[plan.variant].kernel[flavour];
-        UMI_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+        UMI_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit),
                  "cudaFuncSetAttribute");
     }
     return UMI_OK;
