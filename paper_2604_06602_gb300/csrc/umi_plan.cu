@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdlib>
 #include <fstream>
 #include <map>
@@ -233,7 +234,24 @@ umi_status make_plan(int W, int64_t positions, Plan *plan)
 // 48.  Bands of at most G steps per warp take the shortest chain that gives
 // every resident warp one tile (chains up to G are bank-conflict free too):
 // one curve of 18,000 samples at W = 721 43 us at a chain of 16, 33 at 8, 31 at
-// 4, 35 at 2 (two tiles for some warps).
+// 4, 35 at 2 (two tiles for some warps).  The MAD's one-window kernel of the paired
+// variant takes the paired one's chain: 25.4 us at 6, 26.8 at its own 4.
+//
+// That cost knows no whole rounds, which decide where every warp gets a few tiles
+// of equal length.  So in groups of 1 and 32 lanes, and of 2 for one curve, the
+// result is held against the band's own chain and the chain of one tile per
+// resident warp, by the steps of the busiest SM: one curve's tiles come in whole
+// CTAs, as do a batch's that are all resident at once (its curves end unevenly,
+// 20 %), and the last of them leave the SM partly filled.  Its warps' steps are
+// faster then, nearly in proportion, but not in the variants of 8 warps per SM;
+// and a start costs half a step in groups of one or two lanes.  A chain that is
+// 6 % shorter by this count is taken: one curve of 300,000 samples at W = 4095
+// 1.67 ms at 32, 1.48 at the band's 124 (two full rounds); one of 160,000 at W = 51
+// 21.9 us at 1, 18.3 at 3; three of 118,000 at W = 17 31.7 at 1, 27.3 at 3.  Over
+// 378 launches of 1 to 400 curves at W = 1 to 4095 the time is 2.5 % above the best
+// chain's (geometric mean; without it 4.3 %, at the band's chain 9.9 %) and nowhere
+// above what it is without it.  The other groups' steps do not follow the count
+// (up to 5 % slower by it), nor do the paired windows', which are bound by latency.
 void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
 {
     static const double kStartSteps = 0.75, kTailTiles = 0.35;
@@ -250,7 +268,7 @@ void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
         plan->chain = (int)std::max<int64_t>(1, steps);
         return;
     }
-    const int cap = chain_cap(G);
+    const int cap = chain_cap(G), band_chain = plan->chain;
     double best = 1e300;
     for (int c = chain_at_least(G, 1); c <= cap; c = chain_at_least(G, c + 1)) {
         const double tiles = (double)positions / (groups * c) + 0.5 * (double)n_curves;
@@ -260,6 +278,30 @@ void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
             plan->chain = c;
         }
         if (G >= 32 && c >= 16) c += 7;  // a coarser grid is enough there
+    }
+    if (pairs || (G > 2 && G < 32) || (G == 2 && n_curves > 1)) return;
+    const int64_t cta_warps = plan->threads / 32, sms = warps / (8 * t[plan->variant].minb);
+    const int64_t resident = 8 * t[plan->variant].minb / cta_warps;  // CTAs per SM
+    auto busiest = [&](int c) {
+        const int64_t windows = (int64_t)groups * c;
+        const double tiles = n_curves == 1 ? (double)((positions + windows - 1) / windows)
+                                           : (double)positions / (double)windows + 0.5 * (double)n_curves;
+        double rounds = tiles / (double)warps + kTailTiles;
+        if (n_curves == 1 || tiles <= (double)warps) {
+            const int64_t ctas = ((int64_t)std::ceil(tiles) + cta_warps - 1) / cta_warps;
+            const int64_t k = (ctas + sms - 1) / sms, rest = k % resident;
+            const double idle = t[plan->variant].minb == 1 ? 1.0 : 0.1;  // pace of an empty SM
+            rounds = (double)(k / resident);
+            if (rest) rounds += idle + (1.0 - idle) * (double)rest / (double)resident;
+            if (n_curves > 1) rounds *= 1.2;
+        }
+        return rounds * (c + (G <= 2 ? 0.5 : kStartSteps));
+    };
+    best = 0.94 * busiest(plan->chain);
+    for (int c : {band_chain, chain_at_least(G, steps)}) {
+        if (c > cap || busiest(c) >= best) continue;
+        best = busiest(c);
+        plan->chain = c;
     }
 }
 
