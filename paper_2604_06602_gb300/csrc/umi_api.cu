@@ -40,7 +40,14 @@ umi_status fail_cuda(cudaError_t err, const char *what)
     return err == cudaErrorMemoryAllocation ? UMI_ERR_OOM : UMI_ERR_CUDA;
 }
 
-void clear_error() { t_error.clear(); }
+// Every entry point starts here.  CUDA keeps a refused launch's error for the
+// thread's next cudaGetLastError: the call that met it has reported it, and this
+// call's checks after its own launches must not find it.
+void clear_error()
+{
+    t_error.clear();
+    cudaGetLastError();
+}
 
 #define UMI_CUDA(call, what)                         \
     do {                                             \
