@@ -41,10 +41,6 @@ struct SegmentCount {
 
 namespace {
 
-constexpr int kSegThreads = 1024;
-constexpr int kSegWarps = kSegThreads / 32;
-constexpr int kSegChunk = 64 * kSegThreads;  // one 64-sample word per thread
-
 // bits[w] bit b = flux[32 w + b] is finite (bits past `total` are 0).
 __global__ void validity_bits_kernel(const float *__restrict__ flux, int64_t total,
                                      unsigned *__restrict__ bits)
@@ -73,119 +69,123 @@ __device__ __forceinline__ uint64_t validity_word(const unsigned *__restrict__ b
     return v;
 }
 
-// Start of the open segment: its first sample and the number of valid samples
-// of the curve before it.
+// The open segment's first sample and the number of the curve's valid samples
+// before it.
 struct Open {
     int64_t start;  // -1: none
     int64_t rank;
 };
 
-// Exclusive scans over the CTA's threads, seeded with `carry`; `carry` becomes
-// the value past the last thread.  `sh` holds kSegWarps entries.
-__device__ __forceinline__ int64_t scan_max(int64_t v, int64_t *sh, int64_t &carry)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v = max(v, u);
-    }
-    if (lane == 31) sh[warp] = v;
-    __syncthreads();
-    int64_t before = carry, all = carry;
-    for (int w = 0; w < kSegWarps; ++w) {
-        if (w < warp) before = max(before, sh[w]);
-        all = max(all, sh[w]);
-    }
-    __syncthreads();
-    const int64_t u = __shfl_up_sync(0xffffffffu, v, 1);
-    carry = all;
-    return lane ? max(before, u) : before;
-}
+__device__ __forceinline__ unsigned lanes_below(int lane) { return (1u << lane) - 1u; }
 
-__device__ __forceinline__ int64_t scan_sum(int64_t v, int64_t *sh, int64_t &carry)
+// Highest lane of `mask` (not 0).
+__device__ __forceinline__ int top_lane(unsigned mask) { return 31 - __clz((int)mask); }
+
+// Inclusive sum over the warp.
+__device__ __forceinline__ int warp_scan(int v, int lane)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += u;
     }
-    if (lane == 31) sh[warp] = v;
-    __syncthreads();
-    int64_t before = carry, all = carry;
-    for (int w = 0; w < kSegWarps; ++w) {
-        if (w < warp) before += sh[w];
-        all += sh[w];
-    }
-    __syncthreads();
-    const int64_t u = __shfl_up_sync(0xffffffffu, v, 1);
-    carry = all;
-    return lane ? before + u : before;
+    return v;
 }
 
-// One pass over a curve per CTA, 65,536 samples at a time.  A thread holds the
-// validity of 64 samples; each valid sample that follows a run of at least
-// gap_min missing ones opens a segment and closes the one before it.  Bound
-// by its four block scans per 65,536 samples (a few us), not by its bytes.
-// WRITE: put the kept segments into `table` and their first work items into
-// `first_tile`; else count them.  Copying the mask to the host and scanning it
-// there took 1.2 ms of a 1.74 ms call on 256 Kepler curves of 4k to 70k
-// samples; the whole call now takes 0.54 ms.
-template <bool WRITE>
-__global__ void __launch_bounds__(kSegThreads)
+__device__ __forceinline__ int64_t tiles_of(int64_t len, int tile)
+{
+    return len < INT32_MAX / 2 ? (int64_t)(((uint32_t)len + (uint32_t)tile - 1u) / (uint32_t)tile)
+                               : (len + tile - 1) / tile;
+}
+
+// One pass over a curve per CTA, 64 samples per thread at a time; each valid
+// sample that follows a run of at least gap_min missing ones opens a segment and
+// closes the one before it.  WRITE: put the kept segments into `table` and their
+// first work items into `first_tile` (and clear the work counters); else count
+// them.  Bound by latency, a chunk of samples waiting for the one before: so a
+// thread's place among the others comes from ballots and one shuffle (positions
+// ascend with the lane), every warp reads the other warps' totals itself instead
+// of waiting for one that scans them, positions and counts inside a chunk are 32 bits, the
+// next chunk's mask is loaded ahead, and words without a segment start skip the
+// rest.  Two barriers per chunk to count, three to write.  A chunk of 65,536
+// samples takes 1.9 us per pass (one curve of 1e8 samples; with four scans over
+// the CTA's threads in shared memory 9.5): one curve of 1e7 samples at W = 25 3.38 -> 1.04 ms
+// for the whole call (its mask scanned on the host 1.28), 256 Kepler curves of 4k
+// to 70k 520 -> 490 us.
+template <int WARPS, bool WRITE>
+__global__ void __launch_bounds__(WARPS * 32)
     segment_scan_kernel(const unsigned *__restrict__ bits, const float *flux0,
                         const Curve *__restrict__ curves, const SegmentRule *__restrict__ rules,
                         SegmentCount *__restrict__ counts, Curve *__restrict__ table,
-                        int32_t *__restrict__ first_tile)
+                        int32_t *__restrict__ first_tile, uint32_t *__restrict__ counters, int n_counters)
 {
-    __shared__ int64_t sh[kSegWarps];
-    __shared__ Open sh_open[kSegWarps];
+    constexpr int kChunk = 2048 * WARPS;
+    __shared__ int2 sh_valid[WARPS];  // last valid sample (in the chunk, -1: none) and valid samples per warp
+    __shared__ int2 sh_open[WARPS];   // last segment start (-1: none) and its rank in the chunk
+    __shared__ int2 sh_kept[WARPS];   // kept segments and their tiles
     const Curve cv = curves[blockIdx.x];
     const SegmentRule r = rules[blockIdx.x];
     const int64_t first = cv.flux - flux0;  // the curve's first sample in the mask
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int64_t last_valid = -1;      // carries, the same in every thread
+    const int at = threadIdx.x * 64;        // this thread's samples in the chunk
+    int64_t last_valid = -1;                // carries, the same in every thread
     int64_t rank = 0;
     Open open{-1, 0};
-    int64_t n_seg = 0, n_tiles = 0;
+    int64_t n_seg = 0, n_tiles = 0;         // WRITE: a carry too; else this thread's
+    if constexpr (WRITE)
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_counters; k += gridDim.x * blockDim.x)
+            counters[k] = 0u;
 
-    // Appends the segment [start, end) holding `valid` samples if it is kept.
-    auto close = [&](int64_t start, int64_t end, int64_t valid, int64_t &seg, int64_t &tiles) {
-        if (start < 0 || valid < r.min_seg) return;
-        if constexpr (WRITE) {
-            Curve c = cv;
-            c.flux += start;
-            c.trend += start;
-            c.detr += start;
-            c.n = end - start;
-            table[r.seg_base + seg] = c;
-            first_tile[r.seg_base + seg] = (int32_t)(r.tile_base + tiles);
-        }
-        ++seg;
-        tiles += (end - start + r.tile - 1) / r.tile;
+    // Takes the segment [start, end) holding `valid` samples if it is kept.
+    auto close = [&](const Open &o, int64_t end, int64_t end_rank, auto &&kept) {
+        if (o.start >= 0 && end_rank - o.rank >= r.min_seg) kept(o.start, end);
+    };
+    auto put = [&](int64_t start, int64_t end, int64_t seg, int64_t tiles) {
+        Curve c = cv;
+        c.flux += start;
+        c.trend += start;
+        c.detr += start;
+        c.n = end - start;
+        table[r.seg_base + seg] = c;
+        first_tile[r.seg_base + seg] = (int32_t)(r.tile_base + tiles);
     };
 
-    for (int64_t base = 0; base < cv.n; base += kSegChunk) {
-        const int64_t b0 = base + (int64_t)threadIdx.x * 64;
-        const uint64_t word = validity_word(bits, first + b0, first + cv.n);
-        const int64_t before = scan_max(word ? b0 + 63 - __clzll((long long)word) : -1, sh, last_valid);
-        const int64_t rank0 = scan_sum(__popcll(word), sh, rank);
+    uint64_t word = validity_word(bits, first + at, first + cv.n);
+    for (int64_t base = 0; base < cv.n; base += kChunk) {
+        const uint64_t next = validity_word(bits, first + base + kChunk + at, first + cv.n);
+        // The last valid sample and the valid samples before this word.
+        const int own = word ? at + 63 - __clzll((long long)word) : -1;
+        const unsigned some = __ballot_sync(0xffffffffu, word != 0);
+        const unsigned some_below = some & lanes_below(lane);
+        const int near = __shfl_sync(0xffffffffu, own, some_below ? top_lane(some_below) : 0);
+        const int count = __popcll(word);
+        const int upto = warp_scan(count, lane);
+        int before_rel = some_below ? near : -1, rank_rel = upto - count;
+        int chunk_last = some ? __shfl_sync(0xffffffffu, own, top_lane(some)) : -1;
+        int chunk_rank = __shfl_sync(0xffffffffu, upto, 31);
+        if constexpr (WARPS > 1) {
+            if (lane == 0) sh_valid[warp] = make_int2(chunk_last, chunk_rank);
+            __syncthreads();
+            const int2 w = lane < WARPS ? sh_valid[lane] : make_int2(-1, 0);
+            const unsigned full = __ballot_sync(0xffffffffu, w.x >= 0), full_below = full & lanes_below(warp);
+            const int prev = __shfl_sync(0xffffffffu, w.x, full_below ? top_lane(full_below) : 0);
+            if (!some_below && full_below) before_rel = prev;
+            rank_rel += __reduce_add_sync(0xffffffffu, lane < warp ? w.y : 0);
+            chunk_last = full ? __shfl_sync(0xffffffffu, w.x, top_lane(full)) : -1;
+            chunk_rank = __reduce_add_sync(0xffffffffu, w.y);
+        }
+        const int64_t before = before_rel >= 0 ? base + before_rel : last_valid;
 
-        // Visits this word's segment starts in order, with the open segment
-        // and the last valid sample before each.
-        auto visit = [&](Open &o, auto &&on_start) {
+        // Visits this word's segment starts in order: sample, the end of the
+        // segment before it, and its rank in the chunk.
+        auto visit = [&](auto &&on_start) {
             int64_t lv = before;
             int seen = 0;
             uint64_t w = word;
             while (w) {
                 const int bit = __ffsll((long long)w) - 1;
-                const int64_t i = b0 + bit;
-                if (lv < 0 || i - lv - 1 >= r.gap_min) {
-                    on_start(o, lv + 1, rank0 + seen);
-                    o.start = i;
-                    o.rank = rank0 + seen;
-                }
+                const int64_t i = base + at + bit;
+                if (lv < 0 || i - lv - 1 >= r.gap_min) on_start(at + bit, lv + 1, rank_rel + seen);
                 // On to the end of this run of valid samples.
                 const uint64_t inv = ~(w >> bit);
                 const int run = min(inv ? __ffsll((long long)inv) - 1 : 64, 64 - bit);
@@ -194,53 +194,138 @@ __global__ void __launch_bounds__(kSegThreads)
                 w = bit + run < 64 ? (w >> (bit + run)) << (bit + run) : 0ull;
             }
         };
-        // The open segment before this thread's word: the last start of the
-        // threads before it.
-        Open mine{-1, 0};
-        visit(mine, [](Open &, int64_t, int64_t) {});
-        Open inc = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t us = __shfl_up_sync(0xffffffffu, inc.start, o);
-            const int64_t ur = __shfl_up_sync(0xffffffffu, inc.rank, o);
-            if (lane >= o && inc.start < 0) inc = Open{us, ur};
+        // The open segment before this word: the last start before it.
+        int2 mine = make_int2(-1, 0);
+        visit([&](int start, int64_t, int rk) { mine = make_int2(start, rk); });
+        const unsigned starts = __ballot_sync(0xffffffffu, mine.x >= 0);
+        const unsigned starts_below = starts & lanes_below(lane);
+        int2 pre = make_int2(-1, 0), all = make_int2(-1, 0);
+        if (starts) {
+            const int src = starts_below ? top_lane(starts_below) : 0, top = top_lane(starts);
+            const int px = __shfl_sync(0xffffffffu, mine.x, src), py = __shfl_sync(0xffffffffu, mine.y, src);
+            if (starts_below) pre = make_int2(px, py);
+            all = make_int2(__shfl_sync(0xffffffffu, mine.x, top), __shfl_sync(0xffffffffu, mine.y, top));
         }
-        if (lane == 31) sh_open[warp] = inc;
-        __syncthreads();
-        Open pre = open, all = open;
-        for (int w = 0; w < kSegWarps; ++w) {
-            const Open o = sh_open[w];
-            if (o.start < 0) continue;
-            if (w < warp) pre = o;
-            all = o;
+        if constexpr (WARPS > 1) {
+            if (lane == 0) sh_open[warp] = all;
+            __syncthreads();
+            const int2 w = lane < WARPS ? sh_open[lane] : make_int2(-1, 0);
+            const unsigned full = __ballot_sync(0xffffffffu, w.x >= 0), full_below = full & lanes_below(warp);
+            if (full) {
+                const int src = full_below ? top_lane(full_below) : 0, top = top_lane(full);
+                const int px = __shfl_sync(0xffffffffu, w.x, src), py = __shfl_sync(0xffffffffu, w.y, src);
+                if (!starts_below && full_below) pre = make_int2(px, py);
+                all = make_int2(__shfl_sync(0xffffffffu, w.x, top), __shfl_sync(0xffffffffu, w.y, top));
+            }
         }
-        __syncthreads();
-        {
-            const int64_t us = __shfl_up_sync(0xffffffffu, inc.start, 1);
-            const int64_t ur = __shfl_up_sync(0xffffffffu, inc.rank, 1);
-            if (lane && us >= 0) pre = Open{us, ur};
-        }
-        open = all;
-        // Count this word's kept segments, then (write pass) place them.
-        int64_t seg = 0, tiles = 0;
-        auto count = [&](int64_t start, int64_t end, int64_t valid) {
-            if (start < 0 || valid < r.min_seg) return;
-            ++seg;
-            tiles += (end - start + r.tile - 1) / r.tile;
+        const Open before_word = pre.x >= 0 ? Open{base + pre.x, rank + pre.y} : open;
+        // Closes the segments that end at this word's starts.
+        auto closed = [&](auto &&kept) {
+            if (mine.x < 0) return;
+            Open o = before_word;
+            visit([&](int start, int64_t end, int rk) {
+                close(o, end, rank + rk, kept);
+                o = Open{base + start, rank + rk};
+            });
         };
-        Open o = pre;
-        visit(o, [&](Open &p, int64_t end, int64_t rk) { count(p.start, end, rk - p.rank); });
-        int64_t seg0 = scan_sum(seg, sh, n_seg);
-        int64_t tiles0 = scan_sum(tiles, sh, n_tiles);
         if constexpr (WRITE) {
-            o = pre;
-            visit(o, [&](Open &p, int64_t end, int64_t rk) { close(p.start, end, rk - p.rank, seg0, tiles0); });
+            int seg = 0, tiles = 0;  // the host has checked that a band's tiles fit 32 bits
+            closed([&](int64_t start, int64_t end) {
+                ++seg;
+                tiles += (int)tiles_of(end - start, r.tile);
+            });
+            const bool any = __any_sync(0xffffffffu, seg > 0);
+            const int seg_upto = any ? warp_scan(seg, lane) : 0, tiles_upto = any ? warp_scan(tiles, lane) : 0;
+            int64_t seg0 = n_seg + seg_upto - seg, tiles0 = n_tiles + tiles_upto - tiles;
+            int seg_all = __shfl_sync(0xffffffffu, seg_upto, 31), tiles_all = __shfl_sync(0xffffffffu, tiles_upto, 31);
+            if constexpr (WARPS > 1) {
+                if (lane == 0) sh_kept[warp] = make_int2(seg_all, tiles_all);
+                __syncthreads();
+                const int2 w = lane < WARPS ? sh_kept[lane] : make_int2(0, 0);
+                seg0 += __reduce_add_sync(0xffffffffu, lane < warp ? w.x : 0);
+                tiles0 += __reduce_add_sync(0xffffffffu, lane < warp ? w.y : 0);
+                seg_all = __reduce_add_sync(0xffffffffu, w.x);
+                tiles_all = __reduce_add_sync(0xffffffffu, w.y);
+            }
+            if (seg > 0)
+                closed([&](int64_t start, int64_t end) {
+                    put(start, end, seg0, tiles0);
+                    ++seg0;
+                    tiles0 += tiles_of(end - start, r.tile);
+                });
+            n_seg += seg_all;
+            n_tiles += tiles_all;
+        } else {
+            closed([&](int64_t start, int64_t end) {
+                ++n_seg;
+                n_tiles += tiles_of(end - start, r.tile);
+            });
+        }
+        if (all.x >= 0) open = Open{base + all.x, rank + all.y};
+        if (chunk_last >= 0) last_valid = base + chunk_last;
+        rank += chunk_rank;
+        word = next;
+    }
+    // The segment that the curve's end closes.
+    if constexpr (WRITE) {
+        if (threadIdx.x == 0)
+            close(open, last_valid + 1, rank, [&](int64_t start, int64_t end) { put(start, end, n_seg, n_tiles); });
+    } else {
+        if (threadIdx.x == 0)
+            close(open, last_valid + 1, rank, [&](int64_t start, int64_t end) {
+                ++n_seg;
+                n_tiles += tiles_of(end - start, r.tile);
+            });
+        __shared__ longlong2 sh_sum[WARPS];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            n_seg += __shfl_xor_sync(0xffffffffu, n_seg, o);
+            n_tiles += __shfl_xor_sync(0xffffffffu, n_tiles, o);
+        }
+        if (lane == 0) sh_sum[warp] = make_longlong2(n_tiles, n_seg);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            SegmentCount c{0, 0};
+            for (int w = 0; w < WARPS; ++w) {
+                c.tiles += sh_sum[w].x;
+                c.segments += sh_sum[w].y;
+            }
+            counts[blockIdx.x] = c;
         }
     }
-    if (threadIdx.x == 0) {
-        close(open.start, last_valid + 1, rank - open.rank, n_seg, n_tiles);
-        if constexpr (!WRITE) counts[blockIdx.x] = SegmentCount{n_tiles, n_seg};
-    }
+}
+
+// Arguments of either pass.
+struct ScanArgs {
+    const unsigned *bits;
+    const float *flux;
+    const Curve *curves;
+    const SegmentRule *rules;
+    SegmentCount *counts;   // count pass
+    Curve *table;           // write pass
+    int32_t *first_tile;
+    uint32_t *counters;
+    int n_counters;
+};
+
+template <int WARPS, bool WRITE>
+void launch_scan(int n_curves, cudaStream_t stream, const ScanArgs &a)
+{
+    segment_scan_kernel<WARPS, WRITE><<<n_curves, WARPS * 32, 0, stream>>>(
+        a.bits, a.flux, a.curves, a.rules, a.counts, a.table, a.first_tile, a.counters, a.n_counters);
+}
+
+// One CTA per curve, whose chunk is 2,048 samples per warp: one warp up to two
+// chunks, 8 up to two of theirs, else 32.  Short curves in small CTAs, because an
+// SM holds more of them (200,000 curves of 60 samples: 13.4 ms by 1 warp, 14.4 by
+// 8, 20.7 by 32), long ones in large ones (one of 70,000: 111, 82, 78 us; of 1e6: 677,
+// 225, 167); 2,000 of 5,000 take 623, 625 and 688 us.
+template <bool WRITE>
+void scan_segments(int n_curves, int64_t longest, cudaStream_t stream, const ScanArgs &a)
+{
+    if (longest <= 4096) launch_scan<1, WRITE>(n_curves, stream, a);
+    else if (longest <= 32768) launch_scan<8, WRITE>(n_curves, stream, a);
+    else launch_scan<32, WRITE>(n_curves, stream, a);
 }
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -273,16 +358,26 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
     if (total == 0) return UMI_OK;
     if (!flux || !trend || !detr) return fail(UMI_ERR_INVALID_ARG, "null buffer");
 
-    // The whole curves, by band: segments are planned from the whole curves'
-    // bands, as the plain batched call would plan them.
+    // The curves that can hold a kept segment, by band: segments are planned from
+    // the whole curves' bands, as the plain batched call would plan them.
+    BandSizes sizes;
     std::vector<Curve> curves;
     curves.reserve((size_t)B);
+    int64_t longest = 0;
     for (int32_t b = 0; b < B; ++b) {
         const int64_t o = offsets[b], n = offsets[b + 1] - offsets[b];
-        if (n > 0) curves.push_back(make_curve(flux + o, trend + o, detr + o, n, W[b], p));
+        sizes[std::make_pair((int)W[b], p.scale_mode)] += n;
+        if (n == 0 || n < (sp.min_seg >= 0 ? sp.min_seg : W[b] / 3)) continue;
+        curves.push_back(make_curve(flux + o, trend + o, detr + o, n, W[b], p));
+        longest = std::max(longest, n);
+    }
+    if (curves.empty()) {
+        cudaError_t e = cudaMemsetAsync(trend, 0xff, sizeof(float) * (size_t)total, stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(detr, 0xff, sizeof(float) * (size_t)total, stream);
+        return e == cudaSuccess ? UMI_OK : fail_cuda(e, "segment scan");
     }
     BatchLayout lay;
-    st = build_layout(curves, &lay);
+    st = build_layout(curves, &lay, &sizes);
     if (st != UMI_OK) return st;
     for (const auto &band : lay.bands) {
         st = prepare_kernel(band.plan, band.flavour);
@@ -323,8 +418,8 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
     if (e == cudaSuccess) {
         const int64_t blocks = std::min<int64_t>((words * 32 + 255) / 256, 1 << 16);
         validity_bits_kernel<<<(int)blocks, 256, 0, stream>>>(flux, total, d_bits);
-        segment_scan_kernel<false><<<(int)C, kSegThreads, 0, stream>>>(d_bits, flux, d_curves, d_rules, d_counts,
-                                                                       nullptr, nullptr);
+        scan_segments<false>((int)C, longest, stream,
+                             ScanArgs{d_bits, flux, d_curves, d_rules, d_counts, nullptr, nullptr, nullptr, 0});
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
@@ -378,11 +473,13 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
         memcpy(stage.p + rule_off, rules.data(), C * sizeof(SegmentRule));
         e = cudaMemcpyAsync(d_rules, stage.p + rule_off, C * sizeof(SegmentRule), cudaMemcpyHostToDevice, stream);
         stage.release(stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(dev + sc.counter_off, 0, sc.bytes - sc.counter_off, stream);
         if (e == cudaSuccess) {
-            segment_scan_kernel<true><<<(int)C, kSegThreads, 0, stream>>>(
-                d_bits, flux, d_curves, d_rules, nullptr, reinterpret_cast<Curve *>(dev + sc.curve_off),
-                reinterpret_cast<int32_t *>(dev + sc.tile_off));
+            scan_segments<true>((int)C, longest, stream,
+                                ScanArgs{d_bits, flux, d_curves, d_rules, nullptr,
+                                         reinterpret_cast<Curve *>(dev + sc.curve_off),
+                                         reinterpret_cast<int32_t *>(dev + sc.tile_off),
+                                         reinterpret_cast<uint32_t *>(dev + sc.counter_off),
+                                         (int)out.bands.size()});
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) st = enqueue_bands(out, dev, sc, stream, &launches);
