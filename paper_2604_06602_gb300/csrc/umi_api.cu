@@ -275,7 +275,7 @@ static umi_status detrend_single(const float *flux, int64_t n, int32_t W, const 
 
 // ------------------------------------------------------------- batches --
 umi_status build_layout(const std::vector<Curve> &curves, BatchLayout *layout,
-                        const BandSizes *plan_sizes)
+                        const BandSizes *plan_sizes, bool split)
 {
     int nvar = 0;
     variant_table(&nvar);
@@ -324,7 +324,7 @@ umi_status build_layout(const std::vector<Curve> &curves, BatchLayout *layout,
         int64_t positions = 0;
         for (const Curve &c : cs) positions += c.n;
         Plan plan = plans[std::make_pair(cs.front().W, cs.front().scale_mode)];
-        fit_launch(positions, (int64_t)cs.size(), &plan);
+        fit_launch(positions, (int64_t)cs.size(), &plan, split);
         umi_status st = layout->add_band(plan, std::get<4>(kv.first), cs);
         if (st != UMI_OK) return st;
     }

@@ -69,8 +69,9 @@ int plan_regime(int W, int64_t positions);
 // else the measured rule; the chain shrinks for small bands.
 umi_status make_plan(int W, int64_t positions, Plan *plan);
 // Sets the chain of a launch over `n_curves` curves with `positions` windows in
-// all (results do not depend on it).  Tuned plans keep theirs.
-void fit_launch(int64_t positions, int64_t n_curves, Plan *plan);
+// all (results do not depend on it).  `split`: the curves run in pieces that are
+// not known yet.  Tuned plans keep theirs.
+void fit_launch(int64_t positions, int64_t n_curves, Plan *plan, bool split = false);
 // The plans umi_autotune times for a band of `positions` windows of length W.
 std::vector<Plan> autotune_candidates(int W, int64_t positions);
 // Records a tuned plan for (W, p.regime).
@@ -143,7 +144,7 @@ struct BatchLayout {
     umi_status add_band(const Plan &plan, int flavour, const std::vector<Curve> &cs);
 };
 umi_status build_layout(const std::vector<Curve> &curves, BatchLayout *layout,
-                        const BandSizes *plan_sizes = nullptr);
+                        const BandSizes *plan_sizes = nullptr, bool split = false);
 
 // Device scratch for one batch: [curve table][first tiles][one counter per
 // band], all of it written by the host.

@@ -251,8 +251,10 @@ umi_status make_plan(int W, int64_t positions, Plan *plan)
 // 378 launches of 1 to 400 curves at W = 1 to 4095 the time is 2.5 % above the best
 // chain's (geometric mean; without it 4.3 %, at the band's chain 9.9 %) and nowhere
 // above what it is without it.  The other groups' steps do not follow the count
-// (up to 5 % slower by it), nor do the paired windows', which are bound by latency.
-void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
+// (up to 5 % slower by it), nor do the paired windows', which are bound by latency;
+// and curves that run in pieces (`split`) have tiles of all lengths: one of 1e6 in 90,000
+// segments at W = 25 takes 0.84 ms by the first cost's chain, 1.25 by the count's.
+void fit_launch(int64_t positions, int64_t n_curves, Plan *plan, bool split)
 {
     static const double kStartSteps = 0.75, kTailTiles = 0.35;
     if (plan->tuned) return;
@@ -279,7 +281,7 @@ void fit_launch(int64_t positions, int64_t n_curves, Plan *plan)
         }
         if (G >= 32 && c >= 16) c += 7;  // a coarser grid is enough there
     }
-    if (pairs || (G > 2 && G < 32) || (G == 2 && n_curves > 1)) return;
+    if (split || pairs || (G > 2 && G < 32) || (G == 2 && n_curves > 1)) return;
     const int64_t cta_warps = plan->threads / 32, sms = warps / (8 * t[plan->variant].minb);
     const int64_t resident = 8 * t[plan->variant].minb / cta_warps;  // CTAs per SM
     auto busiest = [&](int c) {

@@ -377,7 +377,7 @@ umi_status detrend_segmented(const float *flux, const int64_t *offsets, const in
         return e == cudaSuccess ? UMI_OK : fail_cuda(e, "segment scan");
     }
     BatchLayout lay;
-    st = build_layout(curves, &lay, &sizes);
+    st = build_layout(curves, &lay, &sizes, /*split=*/true);
     if (st != UMI_OK) return st;
     for (const auto &band : lay.bands) {
         st = prepare_kernel(band.plan, band.flavour);
