@@ -46,8 +46,8 @@ LANES_PER_SM = 128
 # headline workload, from the ncu capture of that workload, valid only while
 # the kernel's code (comments and blank lines removed) hashes to
 # `kernel_sha256`.
-MEASURED_TRAFFIC = {"bytes": 161.98e6,
-                    "kernel_sha256": "89c5bc4b69339e1cac4a4e6f65ea47dca6039b380794ebf688c5a4de46b1539c"}
+MEASURED_TRAFFIC = {"bytes": 161.23e6,
+                    "kernel_sha256": "78b12595120d3a4d1df78397964b84f7af775fa0039bd40966d4fef1fdb0eee3"}
 KERNEL_SOURCE = os.path.join(ROOT, "paper_2604_06602_gb300", "csrc", "umi_kernel.cuh")
 
 

@@ -2,8 +2,9 @@
 // that they can be built and checked on their own (tests build them with
 // AddressSanitizer and UndefinedBehaviorSanitizer):
 //   * the server's first-fit arena allocator (umi_server.cu);
-//   * the gap scan of the segmented entry point (umi_segments.cu), which
-//     reads a 1-bit-per-sample validity mask;
+//   * the gap split's rule in sequential form, over a 1-bit-per-sample validity
+//     mask: a model of the segmented entry point's scan (umi_segments.cu), which
+//     runs on the device and is not this code;
 //   * the server's batching policy: which window length and stream the next
 //     batch takes, and which admitted requests go into it.
 #pragma once

@@ -155,18 +155,6 @@ __device__ __forceinline__ unsigned group_umin(unsigned v)
     }
 }
 
-template <int G>
-__device__ __forceinline__ unsigned group_umax(unsigned v)
-{
-    if constexpr (G == 32) {
-        return __reduce_max_sync(0xffffffffu, v);
-    } else {
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-        return v;
-    }
-}
-
 // d = clamp(a*b + c, 0, 1), NaN -> 0, as one saturating FMA.
 __device__ __forceinline__ float fma_sat(float a, float b, float c)
 {
@@ -361,10 +349,14 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
     return SCALAR ? make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)) : __ffma2_rn(a, b, c);
 }
 
-// Which of the iteration's FMAs are scalar pairs.  The FMA pipe takes two
-// cycles for a packed instruction and one for a scalar one, so the mixes cost
-// the same there, but some are scheduled better.  Each lane split has the mix
-// that its variants like best of 32 (kernel times, all packed against it: W = 25
+// Which of the iteration's FMAs are scalar pairs.  The FMA pipe takes about two
+// cycles for a packed instruction and about one for a scalar one, alone or
+// between packed ones (16 warps per SM: FFMA2 2.18, two FFMA 2.42, FFMA2 and FFMA
+// 3.17, FFMA2 and two FFMA 4.27), so the mixes cost nearly the same there, but
+// some are scheduled better.  Each lane split has the mix that those of its variants
+// that were measured like best of 32; the others, (2,44), (4,38), (8,40), (8,48),
+// (8,56), (16,40), (32,56) and (32,92) on among them, take the mix of the nearest
+// measured one unmeasured (kernel times, all packed against it: W = 25
 // (1,26) 0.576 -> 0.569 ms, W = 49 (1,52) 0.566 -> 0.550, W = 73 (2,38) 0.647 ->
 // 0.633, W = 97 (2,52) 0.662 -> 0.647, W = 217 (4,56) 1.342 -> 1.329, W = 361
 // (8,46) 2.595 -> 2.515, W = 541 (8,68) 1.839 -> 1.829, W = 721 (16,48) 1.807 ->
@@ -396,8 +388,10 @@ enum : int { kFlagDiag = 1, kFlagMad = 2, kFlagMin = 4 };
 // Whether a select may pick a positive sample by its bit patterns
 // (select_rank).  That pass is the shorter one, but the min form's loops of 8
 // lanes up to 46 slots and of long 2-lane windows are scheduled better without
-// it (alpha = 10, 300 curves at W = 361: 2.781 -> 2.729 ms; 495 curves at
-// W = 121: 1.568 -> 1.533 ms); its other variants lose 0.1 to 1 % without it.
+// it (alpha = 10, 300 curves at W = 361, (8,46,2): 2.781 -> 2.729 ms; 495 curves
+// at W = 121, (2,62,2): 1.568 -> 1.533; 618 at W = 97, (2,52,2): 1.674 -> 1.638).
+// The other variants measured lose up to 2 % without it; (2,44), (8,24) and (8,40),
+// which were not, lie on their side by lanes and slots alone.
 __host__ __device__ constexpr bool picks_by_bits(int G, int R, int flags)
 {
     return (flags & kFlagMin) == 0 || !((G == 8 && R <= 46) || (G == 2 && R > 38));

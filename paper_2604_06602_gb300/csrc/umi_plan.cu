@@ -168,7 +168,8 @@ int plan_regime(int W, int64_t positions)
 // Chain for `positions` windows of a band in `regime`: about kWarpsPerSm
 // warps per SM get a tile -- kWarpsPerSmNarrow for groups of one or two lanes
 // in the latency regime, whose chain-start selects (a lane scans its whole
-// window once per bit) cost more than the longer chains they save.
+// window in every pass) cost more than the longer chains they save.  An untuned
+// launch then fits its own (fit_launch).
 static int chain_for(int G, int64_t positions, int regime)
 {
     const int sms = std::max(1, device_info(current_device()).sms);

@@ -92,8 +92,10 @@ const Variant *variant_table(int *count);
 
 // The variant list: (G, R, MINB), ordered by slot capacity G*R; for equal
 // capacity the first entry is the default and the autotuner may pick others.
-// Every slot past W is work for nothing, so the capacities follow each other
-// within about a fifth; and a capacity is cut into as few lanes as 56 to 68
+// Every slot past W is work for nothing, so from 64 to 1,088 slots the capacities
+// follow each other within about a fifth (3 to 21 %); below, with few slots, they
+// step by 23 to 100 %, and from 1,088 to 1,536 (41 %) and 2,176 to 2,944 (35 %)
+// there is none between.  A capacity is cut into as few lanes as 56 to 68
 // slots allow: fewer lanes reduce in fewer steps and serve more windows per
 // warp at the same 16 warps per SM.  ns per window, large bands: W = 73 (2,38)
 // 0.106, (4,20) 0.120, (4,32) 0.176; W = 217 (4,56) 0.289, (8,28) 0.342, (8,46)
@@ -101,7 +103,8 @@ const Variant *variant_table(int *count);
 // (32,128) 5.4.  (2,32,2) and (4,32,2) are there because small bands take the
 // largest register budget among the near capacities and would otherwise skip
 // to the next one; no 32-lane capacity lies between 721 and 1442, where small
-// bands of W = 721 would take it in place of (16,48,2).
+// bands of W = 721 would take it in place of (16,48,2) (latency_variant's "within
+// 2W"), so windows of 1,089 to 1,441 samples run on 1,536 slots.
 #define UMI_VARIANT_LIST(X) \
     X(1, 8, 4)           \
     X(1, 16, 4)          \
